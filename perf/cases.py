@@ -221,3 +221,95 @@ def tolerance(case):
     rows = m if case["kind"] == "layer" else (case["tokens"] + case["block"] - 1) // case["block"]
     words = case["hq"] * rows * ((m + 31) // 32)
     return {"rel": 7e-3, "differ": min(0.5, max(2e-4, 2.5 / words))}
+
+
+def _exact_stats(k, block):
+    """Centroids [hkv, m, d], radii and rescue coefficients [hkv, m] in 64 bits of the keys k [n, hkv, d]."""
+    n = k.shape[0]
+    full = n // block
+    parts = [k[:full * block].double().view(full, block, *k.shape[1:])] if full else []
+    if n > full * block:
+        parts.append(k[full * block:].double().unsqueeze(0))
+    c = torch.cat([p.mean(1) for p in parts])                                              # [m, hkv, d]
+    r = torch.cat([(p - p.mean(1, keepdim=True)).norm(dim=-1).amax(1) for p in parts])     # [m, hkv]
+    lo, hi = torch.quantile(r, 0.5, dim=0), torch.quantile(r, 0.9, dim=0)
+    beta = torch.where(hi > lo, ((r - lo) / torch.where(hi > lo, hi - lo, torch.ones_like(hi))).clamp(0, 1), torch.zeros_like(r))
+    return c.transpose(0, 1), r.t(), beta.t()
+
+
+def _exact_rows(q, k, v, stats, block, first, alphas):
+    """Selection and attention in 64 bits of the query tokens q [nq, hq, d] from query block `first` on: output as q,
+    kept blocks [hq, rows, m].  `stats` None: dense."""
+    nq, hq, d = q.shape
+    n, hkv = k.shape[:2]
+    m, rows = (n + block - 1) // block, (nq + block - 1) // block
+    out = torch.empty(nq, hq, d, dtype=torch.float64, device=q.device)
+    keep = torch.zeros(hq, rows, m, dtype=torch.bool, device=q.device)
+    pos, col = torch.arange(first * block, first * block + nq, device=q.device), torch.arange(n, device=q.device)
+    for h in range(hq):
+        hk = h // (hq // hkv)
+        qh, kh, vh = q[:, h].double() / math.sqrt(d), k[:, hk].double(), v[:, hk].double()
+        for i in range(rows):
+            t0, t1 = i * block, min(nq, (i + 1) * block)
+            at = first + i
+            nb = at + 1
+            if stats is None:
+                rest = kept = None
+                keys, vals, cols = kh[:min(n, nb * block)], vh[:min(n, nb * block)], col[:min(n, nb * block)]
+            else:
+                c, r, beta = (x[hk, :nb] for x in stats)
+                z = qh[t0:t1] @ c.t()
+                zr = z + qh[t0:t1].norm(dim=1, keepdim=True) * (r * beta)
+                sb, sr = torch.logsumexp(z, 0), torch.logsumexp(zr, 0)
+                kept = (sb >= math.log(alphas[0]) + sb.max()) | (sr >= math.log(alphas[1]) + sr.max())
+                kept[0] = kept[at] = True                       # the first block and the query block's own
+                if at == m - 1:                                 # the sequence's last query block keeps all
+                    kept[:] = True
+                keep[h, i, :nb] = kept
+                rest = kept.nonzero()[:, 0]
+                cols = (rest[:, None] * block + torch.arange(block, device=q.device)).flatten()
+                cols = cols[:cols.numel() - max(0, nb * block - n)]          # the last kept block is the query block's own
+                keys, vals = kh[cols], vh[cols]
+            s = qh[t0:t1] @ keys.t()
+            s.masked_fill_(cols[None, :] > pos[t0:t1, None], -math.inf)
+            out[t0:t1, h] = torch.softmax(s, 1) @ vals
+    return out, keep
+
+
+def _words(keep):
+    """[hq, rows, m] kept blocks -> [1, hq, rows, words] 32-bit words, block b in bit b % 32 of word b / 32."""
+    w = (keep.shape[-1] + 31) // 32
+    bits = torch.nn.functional.pad(keep, (0, 32 * w - keep.shape[-1])).view(*keep.shape[:-1], w, 32).long()
+    x = (bits << torch.arange(32, device=keep.device)).sum(-1)
+    return torch.where(x >= 1 << 31, x - (1 << 32), x).int().unsqueeze(0)
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, from their bf16 values on in 64 bits by the paper's formulas; None where that
+    would take longer than about 20 seconds."""
+    kind, n, block = case["kind"], case["n"], case["block"]
+    lens = _lens(case) if kind == "varlen" else [n]
+    m = sum((x + block - 1) // block for x in lens)
+    if (m if kind != "chunk" else (case["tokens"] + block - 1) // block) * case["hq"] > 20000:
+        return None
+    s = prepare(case, seed)
+    if kind == "varlen":
+        outs, dens = [], []
+        for t0, t1 in zip(s["cu"], s["cu"][1:]):
+            q, k, v = (s[x][t0:t1] for x in "qkv")
+            out, keep = _exact_rows(q, k, v, _exact_stats(k, block), block, 0, s["alphas"])
+            outs.append(out)
+            dens.append(keep.sum((1, 2)).double() / (keep.shape[2] * (keep.shape[2] + 1) / 2))
+        return {"out": torch.cat(outs), "density": torch.stack(dens)}
+    q, k, v = (s[x][0] for x in "qkv")
+    if kind == "dense":
+        return {"out": _exact_rows(q, k, v, None, block, 0, None)[0].unsqueeze(0)}
+    c, r, beta = _exact_stats(k, block)
+    first = case["start"] if kind == "chunk" else 0
+    out, keep = _exact_rows(q, k, v, (c, r, beta), block, first, s["alphas"])
+    rows = keep.shape[1]
+    density = keep.sum((1, 2)).double() / (rows * first + rows * (rows + 1) / 2)
+    res = {"out": out.unsqueeze(0), "mask": _words(keep), "density": density.unsqueeze(0)}
+    if kind == "layer":
+        res.update(centroid=c.unsqueeze(0), radius=r.unsqueeze(0), beta=beta.unsqueeze(0))
+    return res
