@@ -63,6 +63,9 @@ size_t select_box_workspace_bytes(const Dims& x);
 // TMA tensor map over a bf16 [L][N][H][d] tensor with arbitrary (16-byte aligned) strides; box = box_d x box_t.
 rbs_status make_tmap_lthd(::CUtensorMap_st* out, const void* ptr, int L, int N, int H, int d, int64_t sb, int64_t st,
                           int64_t sh, int box_d, int box_t, bool swizzle128);
+// One box = box_t tokens x all kHeadDim columns of one head, as 128-byte-swizzled panels of 64 columns.
+rbs_status make_tmap_panels(::CUtensorMap_st* out, const void* ptr, int L, int N, int H, int64_t sb, int64_t st, int64_t sh,
+                            int box_t);
 rbs_status make_tmap_2d(::CUtensorMap_st* out, const void* ptr, int64_t rows, int cols, int box_cols, int box_rows);
 // Number of SMs of the current device (looked up once per device).
 int sm_count();

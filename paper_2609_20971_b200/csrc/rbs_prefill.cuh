@@ -16,6 +16,7 @@ struct PrefillParams {
   int M, W, L, Hq, G, N;
   int R;   // 128-row tiles per block (tensor-core path): block / 128
   int q0, Mq, Nq;   // this call's queries: first query block (global index), number of blocks, number of tokens
+  int mask_heads;   // heads that share one mask row: 1, or 2 (the row of the first head of each pair is read)
   int band_rows;    // 128-row query tiles per band of the tile order (tensor-core path)
   float scale_log2;
   // Row-length-aware schedule (null: tiles in their static order, one CTA per tile).  One int4 per CTA:
@@ -67,7 +68,7 @@ __device__ __forceinline__ int next_kb(const uint32_t* __restrict__ row, int cur
 // of the tensor-core kernels).
 constexpr float kSumLimit = 16384.0f;
 
-rbs_status launch_prefill_pair(const PrefillParams& p, const rbs_tensor& Q, const rbs_tensor& K, const rbs_tensor& V, int Hkv,
-                               int mode, cudaStream_t s);
+rbs_status launch_prefill_duo(const PrefillParams& p, const rbs_tensor& Q, const rbs_tensor& K, const rbs_tensor& V, int Hkv,
+                              bool blocks64, long long n_items, cudaStream_t s);
 
 }  // namespace rbs

@@ -1,0 +1,762 @@
+// Block-sparse (and dense) causal attention on the 5th-generation tensor cores: two query tiles per SM that share one
+// S accumulator.
+//
+// Per 128-key step of a 128-row query tile:
+//   S[128 q x 128 keys] = Q K^T       (both operands from shared memory, 8 tcgen05.mma of K = 16)
+//   P = 2^(S scale - m)               (64 keys of one query row per thread, lazily updated running maximum m of the row)
+//   O[128 q x 128 d]   += P V         (P from tensor memory, V from shared memory, 8 MMAs)
+// One persistent CTA per SM works on two tiles at a time ("slots" A and B), each with its own stream of K/V tiles.
+// Tensor memory (512 columns): O_A 128 | O_B 128 | S 128 | P_A 64 | P_B 64 (bf16 pairs).  There is ONE S accumulator:
+// the softmax threads copy S into registers first (64 each) and hand the accumulator back at once, so the Q K^T of one
+// slot runs under the exponentials of the other and, because P has columns of its own, neither waits for the P V product
+// before it.  (Before: two CTAs per SM with S and O each and P written over S, so that a tile's Q K^T had to follow its
+// P V and the two tiles' softmaxes ran in phase, the tensor core idle meanwhile.)  Launched back to back, dense attention
+// over 32K tokens and 32 heads takes 7.1 ms = 1,240 TFLOP/s instead of 7.8, the 128K layer at 8 % density 9.7 ms instead
+// of 10.8, the 64-head layer at blocks of 64 24.8 ms instead of 30.5; the launches run at the power cap.
+//
+// Warps 0-7 / 8-15: softmax of slot A / B; the first four warps of a slot take keys 0-63 of a step, the others keys 64-127
+// of the same rows (four warps per scheduler hide one another's tensor-memory accesses and barriers behind the exp unit).
+// Warps 16 / 17: TMA producer of slot A / B.  Warps 18 / 19: MMA issuers of both slots, in turns: warp 18 issues Q K^T of
+// a slot's next step and tells warp 19 to issue P V of its current one behind it, so that P V covers the time from the end
+// of Q K^T until S has been read.  (Two warps, because a wait between two batches of MMAs of one warp costs the tensor
+// core 150 - 250 cycles.)  Warp 19 also owns the tensor-memory allocation.
+// K/V in shared memory per slot: K panel 0 twice, K panel 1 (16 KB each), V (32 KB).
+// Tiles are handed out in grid order (the grid has one CTA per tile): a slot that needs another tile cancels the launch
+// of a CTA that has not started yet and takes its place, so the order of the tiles is the grid's, no counter in global
+// memory is needed, and a tile's epilogue and the start of the next one pass under the other slot's work.
+#include <type_traits>
+
+#include "rbs_prefill.cuh"
+#include "rbs_score.cuh"
+
+namespace rbs {
+
+constexpr int kDuoThreads = 640;
+constexpr uint32_t kDuoStage = 16384;          // one K panel or V half
+constexpr int kDuoStages = 5;                 // per slot: K panel 0 (even / odd steps), K panel 1, V (two)
+constexpr uint32_t kDuoPanel = 128 * 128;     // 128 rows x 64 bf16 columns
+constexpr uint32_t kDuoTile = 2 * kDuoPanel;  // one Q tile
+
+// What the producer tells the MMA issuer and the softmax warps about a step (ring of four entries per slot).
+// Blocks of 128 and more: bit 0: the step's keys are the tile's diagonal sub-block.  Blocks of 64: bits 0-3 describe the
+// step's first key block, bits 4-7 its second (bit 0 / 1: selected by query block A / B of the tile, bit 2 / 3: it is
+// the diagonal block of A / B).
+enum : uint32_t { kStepLast = 1u << 8, kStepOneHalf = 1u << 9, kStepExit = 1u << 31 };
+enum : int { kTileExit = 1, kTileEmpty = 2 };
+struct DuoTileInfo { int Tl, h, l, flags; };
+
+// mbar_wait (rbs_sm100.cuh) for this kernel: the waiting thread is suspended for up to kWaitHintNs per probe instead of
+// probing all the time (twenty warps share the issue slots with the exponentials), and the loop is a handful of
+// instructions without divergence handling.  Bounded: about a second in all, then `code` goes to the status word.
+constexpr uint32_t kWaitHintNs = 20000, kWaitProbes = 50000;
+__device__ __forceinline__ bool duo_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .u32 c;\n\t"
+      "mov.u32 c, 0;\n"
+      "WAIT:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "@p bra.uni DONE;\n\t"
+      "add.u32 c, c, 1;\n\t"
+      "setp.lt.u32 p, c, %4;\n\t"
+      "@p bra.uni WAIT;\n\t"
+      "setp.ne.u32 p, 0, 0;\n"
+      "DONE:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "n"(kWaitHintNs), "n"(kWaitProbes) : "memory");
+  if (ok == 0u) atomicCAS(status, 0u, code);
+  return ok != 0u;
+}
+// one arrival by a converged warp
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}"
+      ::"r"(bar) : "memory");
+}
+// one thread of a converged warp writes a word, then arrives
+__device__ __forceinline__ void warp_tell(uint32_t word, uint32_t value, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e st.shared.u32 [%0], %1;\n\t"
+      "@e mbarrier.arrive.shared::cta.b64 _, [%2];\n\t}"
+      ::"r"(word), "r"(value), "r"(bar) : "memory");
+}
+
+// An mbarrier probe that does not wait.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0u;
+}
+
+// Walks the steps of one tile.  KB = 128: every step is one selected 128-key sub-block of the tile's mask row.
+// KB = 64: the tile holds two consecutive query blocks of 64 (rows 0-63: block iA, rows 64-127: iB = iA + 1), each with
+// its own mask row; a step is two consecutive key blocks of the UNION of the two rows.
+template <int KB>
+struct StepWalk;
+
+template <>
+struct StepWalk<128> {
+  const uint32_t* row; int i, R, T, Tw, cur;
+  __device__ __forceinline__ void start(int kb0) { cur = next_kb(row, kb0, i, R, Tw); }
+  __device__ __forceinline__ bool any() const { return cur >= 0; }
+  // the current step: first key row of its two halves of 64 keys, flags; then moves on
+  __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
+    r0 = cur * 128; r1 = r0 + 64;
+    uint32_t f = cur == T ? 1u : 0u;
+    cur = next_kb(row, cur, i, R, Tw);
+    if (cur < 0) f |= kStepLast;
+    return f;
+  }
+};
+
+template <>
+struct StepWalk<64> {
+  const uint32_t* rowA; const uint32_t* rowB;   // mask rows of the two query blocks (rowB null: no second block)
+  int iA, iB, cur;
+  __device__ __forceinline__ int next(int from) const {   // next key block after `from` selected by either row, or -1
+    const int last = rowB ? iB : iA;
+    int b = from + 1;
+    while (b <= last) {
+      const int w = b >> 5;
+      uint32_t u = __ldg(rowA + w);
+      if (((w + 1) << 5) - 1 > iA) u = (w << 5) > iA ? 0u : (u & (0xffffffffu >> (31 - (iA & 31))));
+      if (rowB) {
+        uint32_t v = __ldg(rowB + w);
+        if (((w + 1) << 5) - 1 > iB) v = (w << 5) > iB ? 0u : (v & (0xffffffffu >> (31 - (iB & 31))));
+        u |= v;
+      }
+      u >>= (b & 31);
+      if (u) return b + __ffs(u) - 1;
+      b = (b | 31) + 1;
+    }
+    return -1;
+  }
+  __device__ __forceinline__ uint32_t flags(int b) const {
+    uint32_t f = 0;
+    if (b <= iA && ((__ldg(rowA + (b >> 5)) >> (b & 31)) & 1u)) f |= 1u;
+    if (rowB && b <= iB && ((__ldg(rowB + (b >> 5)) >> (b & 31)) & 1u)) f |= 2u;
+    if (b == iA) f |= 4u;
+    if (b == iB) f |= 8u;
+    return f;
+  }
+  __device__ __forceinline__ void start(int) { cur = next(-1); }
+  __device__ __forceinline__ bool any() const { return cur >= 0; }
+  __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
+    r0 = cur * 64;
+    uint32_t f = flags(cur);
+    const int b1 = next(cur);
+    if (b1 < 0) { cur = -1; return f | kStepLast | kStepOneHalf; }
+    r1 = b1 * 64;
+    f |= flags(b1) << 4;
+    cur = next(b1);
+    if (cur < 0) f |= kStepLast;
+    return f;
+  }
+};
+
+template <int KB, bool SCHED>
+__global__ void __launch_bounds__(kDuoThreads, 1)
+prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
+                   const PrefillParams p, unsigned int* status) {
+  static_assert(KB == 128 || (KB == 64 && !SCHED), "the schedule exists for blocks of 128 and 256");
+  constexpr uint32_t kIdescQK = idesc_bf16_f32(128, 128, false);
+  constexpr uint32_t kIdescPV = idesc_bf16_f32(128, 128, true);
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* sQ = smem;                    // [slot][kDuoTile]
+  unsigned char* sKV = smem + 2 * kDuoTile;    // [slot][kDuoStages][kDuoStage]
+  __shared__ __align__(16) uint32_t s_clc[4];
+  // per slot.  k: the K of an even / odd step is there; in: P and V are there (eight softmax warps and the producer
+  // arrive); s: S is there, K is free; pv: P V is done, P and V are free (in, pv: with blocks of 64 one per key block); tile / tdone: a tile has been announced / its
+  // output is out.  sfree: S has been read into registers; turn: messages of warp 18 to warp 19
+  __shared__ __align__(8) uint64_t bar_k[2][2], bar_in[2][2], bar_s[2], bar_pv[2][2], bar_sfree, bar_turn[8];
+  __shared__ __align__(8) uint64_t bar_q[2], bar_tile[2], bar_tdone[2], bar_clc;
+  __shared__ float s_xch[2][2][128];             // [slot][key half][row]: maxima, row sums for the other key half
+  __shared__ uint32_t s_step[2][4], s_turn[8];   // turn: the slot whose P V is due
+  __shared__ DuoTileInfo s_tile[2];
+  __shared__ int s_part[2];
+  __shared__ uint32_t s_tmem, s_lock, s_clc_phase, s_no_more;
+
+  const int tid = threadIdx.x, lane = tid & 31;
+  // uniform for the compiler: the roles then run on uniform registers and branches (20 % less code, 55 instead of 128 moves
+  // to uniform registers per step)
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+
+  if (tid == 0) {
+    for (int x = 0; x < 2; ++x) {
+      for (int k = 0; k < 2; ++k) {
+        mbar_init(smem_u32(&bar_k[x][k]), 2);
+        mbar_init(smem_u32(&bar_in[x][k]), 9); mbar_init(smem_u32(&bar_pv[x][k]), 1);
+      }
+      mbar_init(smem_u32(&bar_s[x]), 1); 
+      mbar_init(smem_u32(&bar_q[x]), 1); mbar_init(smem_u32(&bar_tile[x]), 1); mbar_init(smem_u32(&bar_tdone[x]), 1);
+    }
+    for (int k = 0; k < 8; ++k) mbar_init(smem_u32(&bar_turn[k]), 1);
+    mbar_init(smem_u32(&bar_sfree), 8);
+    mbar_init(smem_u32(&bar_clc), 1);
+    s_lock = 0; s_clc_phase = 0; s_no_more = 0;
+    mbar_fence_init();
+  }
+  if (warp == 19) tmem_alloc(smem_u32(&s_tmem), 512);
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = s_tmem;
+  const uint32_t tmem_s = tmem + 256;
+  const int Hkv = p.Hq / p.G;
+
+  if (warp >= 16) reg_dealloc<64>();
+  if (warp == 16 || warp == 17) {
+    // ------------------------------- TMA producer of one slot -------------------------------
+    if (lane == 0) {
+      const int x = warp - 16;
+      if (x == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmO); } else { tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); }
+      // the next tile of the grid, or -1: two threads of the CTA share one request at a time; a request that finds no
+      // CTA left to cancel is the last one made
+      auto fetch = [&]() -> int {
+        bool locked = false;
+#pragma unroll 1
+        for (uint32_t it = 0; it < kSpinLimit; ++it) {
+          if (atomicCAS(&s_lock, 0u, 1u) == 0u) { locked = true; break; }
+          if (it > 64) __nanosleep(64);
+          if ((it & 255u) == 255u && *reinterpret_cast<volatile unsigned int*>(status) != 0u) break;
+        }
+        if (!locked) { atomicCAS(status, 0u, static_cast<unsigned int>(kWaitStageFree)); return -1; }
+        __threadfence_block();
+        int got = -1;
+        if (*reinterpret_cast<volatile uint32_t*>(&s_no_more) == 0u) {
+          const uint32_t ph = *reinterpret_cast<volatile uint32_t*>(&s_clc_phase);
+          const uint32_t resp = smem_u32(s_clc), bar = smem_u32(&bar_clc);
+          fence_proxy_async_smem();                 // the last response has been read
+          mbar_arrive_expect_tx(bar, 16);
+          asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                       ::"r"(resp), "r"(bar) : "memory");
+          uint32_t ok = 0, cx = 0;
+          if (duo_wait(bar, ph, status, kWaitTmaFull)) {
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+                "ld.shared.b128 r, [%2];\n\t"
+                "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t"
+                "mov.u32 %1, 0;\n\t"
+                "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n\t}"
+                : "=r"(ok), "=r"(cx) : "r"(resp) : "memory");
+          }
+          if (ok) got = static_cast<int>(cx);
+          else s_no_more = 1u;
+          s_clc_phase = ph ^ 1u;
+        }
+        __threadfence_block();
+        atomicExch(&s_lock, 0u);
+        return got;
+      };
+      const uint64_t pol_q = make_policy_evict_first();
+      const uint32_t q_dst = smem_u32(sQ) + x * kDuoTile, kv_dst = smem_u32(sKV) + x * kDuoStages * kDuoStage;
+      uint32_t nk = 0, nv = 0;   // steps whose K / V has been requested
+      uint32_t pub = 0;          // tiles announced so far
+      bool ok = true;
+      // (The wait for a phase before the first one passes: its parity is the one before phase 0.)
+      // In the order in which the tensor core frees the buffers: Q K^T of a step, then P V of the step before it.  Every
+      // phase of s and pv is waited for once and in turn.
+      auto load_k = [&](int r0, int r1, uint32_t info, int hk, int l) {
+        s_step[x][nk & 3] = info;
+        const uint32_t bar = smem_u32(&bar_k[x][nk & 1]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          // panel 0 of this parity was freed by the step before last, whose phase was waited for with the last panel 1
+          if (c == 1) ok = duo_wait(smem_u32(&bar_s[x]), (nk - 1) & 1, status, kWaitStageFree);
+          if (!ok) return;
+          const uint32_t dst = kv_dst + (c == 0 ? (nk & 1) : 2) * kDuoStage;
+          if (KB == 128) {
+            mbar_arrive_expect_tx(bar, kDuoStage);
+            tma_load_4d(dst, &tmK, bar, c * 64, hk, r0, l);
+          } else {
+            const bool two = (info & kStepOneHalf) == 0u;
+            mbar_arrive_expect_tx(bar, two ? kDuoStage : kDuoStage / 2);
+            tma_load_4d(dst, &tmK, bar, c * 64, hk, r0, l);
+            if (two) tma_load_4d(dst + kDuoStage / 2, &tmK, bar, c * 64, hk, r1, l);
+          }
+        }
+        ++nk;
+      };
+      auto load_v = [&](int r0, int r1, uint32_t info, int hk, int l) {
+        const uint32_t dst = kv_dst + 3 * kDuoStage;
+#pragma unroll
+        for (int u = 0; u < (KB == 128 ? 1 : 2); ++u) {
+          ok = ok && duo_wait(smem_u32(&bar_pv[x][u]), (nv - 1) & 1, status, kWaitStageFree);
+          if (!ok) return;
+          const uint32_t bar = smem_u32(&bar_in[x][u]);
+          if (u == 1 && (info & kStepOneHalf)) {
+            mbar_arrive(bar);
+          } else {
+            mbar_arrive_expect_tx(bar, KB == 128 ? 2 * kDuoStage : kDuoStage);
+            tma_load_5d(dst + u * kDuoStage, &tmV, bar, 0, hk, u == 0 ? r0 : r1, l, 0);
+          }
+        }
+        ++nv;
+      };
+      const int per_band_kv = SCHED ? p.items_per_group : p.band_rows * p.G;
+      const int per_band = p.L * Hkv * per_band_kv;
+      const int n_rows = KB == 128 ? p.Mq * p.R : (p.Mq + 1) / 2;    // 128-row tiles of the call
+      // -2: to be fetched; a launch in which a wait has given up is lost: CTAs that start after that do nothing
+      int w = *reinterpret_cast<volatile unsigned int*>(status) != 0u ? -1 : x == 0 ? static_cast<int>(blockIdx.x) : -2;
+#pragma unroll 1
+      while (ok) {
+        if (w == -2) w = fetch();
+        if (w < 0) break;
+        // Tile order: the query tiles are cut into bands of band_rows consecutive tiles, the last (longest) band first;
+        // inside a band one (batch, KV head) at a time, inside it longest rows first, the G query heads of the group
+        // together.  All tiles in flight then read the K/V of one KV head (64 MiB at 128K tokens), which stays in L2;
+        // with all KV heads interleaved the K/V tiles of a 128K layer (256 MiB) were re-read from DRAM many times.
+        // The bands keep the very long rows (the dense rows of the last query blocks) of every KV head near the start
+        // of the launch.  SCHED: the item list of plan_rows_kernel instead: the same order, long rows cut into parts.
+        const int band = w / per_band, rem_band = w % per_band;
+        const int kvid = rem_band / per_band_kv;
+        int rem = rem_band % per_band_kv;
+        int4 item = make_int4(0, 0, 0x7fffffff, -1);
+        if (SCHED) { item = __ldg(p.items + w); rem = item.x; }
+        w = -2;
+        const int l = kvid / Hkv, hk = kvid % Hkv;
+        const int Tl = n_rows - 1 - (band * p.band_rows + rem / p.G);
+        if ((SCHED && item.x < 0) || Tl < 0 || Tl * 128 >= p.Nq) continue;   // no such tile
+        const int h = hk * p.G + rem % p.G;
+        StepWalk<KB> walk;
+        if constexpr (KB == 128) {
+          const int T = p.q0 * p.R + Tl, i = T / p.R;
+          if (!RBS_DBG_OK(i >= p.q0 && i - p.q0 < p.Mq && h < p.Hq && l < p.L && T < p.M * p.R, status, kDbgPrefillTile)) break;
+          walk.row = p.mask ? p.mask + ((static_cast<int64_t>(l) * p.Hq + h - rem % p.G % p.mask_heads) * p.Mq + (i - p.q0)) * p.W : nullptr;
+          walk.i = i; walk.R = p.R; walk.T = T;
+          walk.Tw = SCHED ? min(T, item.z - 1) : T;
+          walk.start(SCHED ? item.y - 1 : -1);
+        } else {
+          walk.iA = p.q0 + 2 * Tl; walk.iB = walk.iA + 1;
+          walk.rowA = p.mask + ((static_cast<int64_t>(l) * p.Hq + h) * p.Mq + 2 * Tl) * p.W;
+          walk.rowB = (2 * Tl + 1 < p.Mq) ? walk.rowA + p.W : nullptr;
+          walk.start(-1);
+        }
+        const bool empty = !walk.any();
+        int r0 = 0, r1 = 0, v0 = 0, v1 = 0;
+        uint32_t info = 0, vinfo = 0;
+#pragma unroll 1
+        for (bool begin = true;; begin = false) {   // the K of a step in front of the V of the step before it
+          if (begin ? !empty : !(vinfo & kStepLast)) {
+            info = walk.take(r0, r1);
+            if (!RBS_DBG_OK(r0 < p.N, status, kDbgPrefillBlock)) { ok = false; break; }
+            load_k(r0, r1, info, hk, l);
+          }
+          if (begin) {
+            // the slot's Q buffer (also the staging buffer of its output) and tile record are free once its last tile is done
+            if (ok) ok = duo_wait(smem_u32(&bar_tdone[x]), (pub - 1) & 1, status, kWaitStageFree);
+            if (!ok) break;
+            s_tile[x].Tl = Tl; s_tile[x].h = h; s_tile[x].l = l; s_tile[x].flags = empty ? kTileEmpty : 0;
+            if (SCHED) s_part[x] = item.w;
+            mbar_arrive(smem_u32(&bar_tile[x]));
+            ++pub;
+            if (empty) break;
+            // Q is read exactly once per launch: evict-first, so that it does not push the K/V in flight out of L2
+            mbar_arrive_expect_tx(smem_u32(&bar_q[x]), kDuoTile);
+            tma_load_4d_hint(q_dst, &tmQ, smem_u32(&bar_q[x]), 0, h, Tl * 128, l, pol_q);
+            tma_load_4d_hint(q_dst + kDuoPanel, &tmQ, smem_u32(&bar_q[x]), 64, h, Tl * 128, l, pol_q);
+          } else if (ok) {
+            load_v(v0, v1, vinfo, hk, l);
+          }
+          if (!ok || (!begin && (vinfo & kStepLast))) break;
+          v0 = r0; v1 = r1; vinfo = info;
+        }
+      }
+      // no tile left: the issuer learns it from a step, the softmax warps from a tile
+      if (ok) {
+        s_step[x][nk & 3] = kStepExit;
+        mbar_arrive(smem_u32(&bar_k[x][nk & 1]));
+        mbar_arrive(smem_u32(&bar_k[x][nk & 1]));
+        ok = duo_wait(smem_u32(&bar_tdone[x]), (pub - 1) & 1, status, kWaitStageFree);
+        if (ok) {
+          s_tile[x].flags = kTileExit;
+          mbar_arrive(smem_u32(&bar_tile[x]));
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 18) {
+    // ------------------------------- MMA issuer: Q K^T -------------------------------
+    // The whole warp runs in lock step and one elected lane issues each tcgen05 instruction; the operand descriptors are
+    // constants of each copy of the code (one that changes has to be moved to uniform registers for every MMA).
+    const uint64_t dq = smem_desc_sw128(smem_u32(sQ), 16, 1024), dk = smem_desc_sw128(smem_u32(sKV), 16, 1024);
+    constexpr uint64_t kStage16 = kDuoStage >> 4;
+    uint32_t n[2] = {0u, 0u}, tiles[2] = {0u, 0u};   // steps issued, tiles begun
+    bool mid[2] = {false, false};                    // inside a tile: P V of step n - 1 is due
+    bool last[2] = {false, false};                   // step n - 1 is its tile's last one
+    bool done[2] = {false, false};
+    uint32_t uses = 0, turns = 0;                    // of S; messages to warp 19
+    bool ok = true;
+    auto tell = [&](uint32_t what) {                 // the slot whose P V is due (2: no more)
+      warp_tell(smem_u32(&s_turn[turns & 7]), what, smem_u32(&bar_turn[turns & 7]));
+      ++turns;
+    };
+    // One turn of slot X; false if it has nothing to do now.  Between two tiles a slot never holds up the other one.
+    auto turn = [&](auto slot) -> bool {
+      constexpr int X = decltype(slot)::value;
+      constexpr uint64_t kKV = static_cast<uint64_t>(X * kDuoStages) * kStage16, kQ = static_cast<uint64_t>(X) * (kDuoTile >> 4);
+      if (done[X]) return false;
+      if (mid[X] && last[X]) {
+        tell(X);
+        mid[X] = false;
+        return true;
+      }
+      const uint32_t kbar = smem_u32(&bar_k[X][n[X] & 1]), kph = (n[X] >> 1) & 1;
+      if (mid[X]) {
+        ok = __all_sync(0xffffffffu, duo_wait(kbar, kph, status, kWaitTmaFull));
+        if (!ok) return false;
+      } else if (!__all_sync(0xffffffffu, mbar_test(kbar, kph))) {
+        return false;
+      }
+      const uint32_t info = *reinterpret_cast<volatile uint32_t*>(&s_step[X][n[X] & 3]);
+      if (!mid[X]) {
+        if (info & kStepExit) { done[X] = true; return true; }
+        if (!__all_sync(0xffffffffu, mbar_test(smem_u32(&bar_q[X]), tiles[X] & 1))) return false;
+        ++tiles[X];
+      }
+      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_sfree), (uses - 1) & 1, status, kWaitTmemFree));
+      if (!ok) return false;
+      tc_fence_after_sync();
+      if (n[X] & 1) mma_ss_k64_commit_elect(tmem_s, dq + kQ, dk + kKV + kStage16, kIdescQK, 0, 0);
+      else mma_ss_k64_commit_elect(tmem_s, dq + kQ, dk + kKV, kIdescQK, 0, 0);
+      if (mid[X]) tell(X);             // by the time warp 19 has seen it, the rest of Q K^T is in the tensor core's queue
+      mma_ss_k64_commit_elect(tmem_s, dq + kQ + (kDuoPanel >> 4), dk + kKV + 2 * kStage16, kIdescQK, smem_u32(&bar_s[X]), 1);
+      ++uses;
+      ++n[X];
+      mid[X] = true;
+      last[X] = (info & kStepLast) != 0u;
+      return true;
+    };
+    uint32_t idle = 0;
+#pragma unroll 1
+    while (ok && !(done[0] && done[1])) {
+      const bool a = turn(std::integral_constant<int, 0>());
+      const bool b = ok && turn(std::integral_constant<int, 1>());
+      if (a || b) { idle = 0; continue; }
+      if (++idle > 2048) __nanosleep(64);
+      if ((idle & 255u) == 255u && (*reinterpret_cast<volatile unsigned int*>(status) != 0u || idle >= kSpinLimit)) {
+        atomicCAS(status, 0u, static_cast<unsigned int>(kWaitTmaFull));
+        ok = false;
+      }
+      ok = __all_sync(0xffffffffu, ok);
+    }
+    if (ok) tell(2u);
+    __syncwarp();
+  } else if (warp == 19) {
+    // ------------------------------- MMA issuer: P V -------------------------------
+    // V: two panels of 64 columns x 128 keys (blocks of 64: two blocks of two panels x 64 keys)
+    const uint64_t dv = smem_desc_sw128(smem_u32(sKV), KB == 128 ? kDuoStage : kDuoStage / 2, 1024);
+    constexpr uint64_t kStage16 = kDuoStage >> 4, kHalf16 = (KB == 128 ? 4 * 2048 : kDuoStage) >> 4;
+    uint32_t n[2] = {0u, 0u};                        // steps issued
+    bool first[2] = {true, true};                    // the next step is its tile's first: O is overwritten
+    bool ok = true;
+    auto product = [&](auto slot) {
+      constexpr int X = decltype(slot)::value;
+      constexpr uint64_t kV = static_cast<uint64_t>(X * kDuoStages + 3) * kStage16;
+      const uint32_t info = *reinterpret_cast<volatile uint32_t*>(&s_step[X][n[X] & 3]);
+      const uint32_t ph = n[X] & 1;
+      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_in[X][0]), ph, status, kWaitPReady));
+      if (!ok) return;
+      tc_fence_after_sync();
+      mma_ts_k64_elect(tmem + X * 128, tmem + 384 + X * 64, dv + kV, kIdescPV, 2048 >> 4, !first[X], KB == 64 ? smem_u32(&bar_pv[X][0]) : 0u);
+      if (KB == 64) {
+        ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_in[X][1]), ph, status, kWaitPReady));
+        if (!ok) return;
+        tc_fence_after_sync();
+      }
+      if (KB == 64 && (info & kStepOneHalf)) mma_commit_elect(smem_u32(&bar_pv[X][1]));
+      else mma_ts_k64_elect(tmem + X * 128, tmem + 384 + X * 64 + 32, dv + kV + kHalf16, kIdescPV, 2048 >> 4, 1, smem_u32(&bar_pv[X][KB == 64 ? 1 : 0]));
+      first[X] = (info & kStepLast) != 0u;
+      ++n[X];
+    };
+#pragma unroll 1
+    for (uint32_t turns = 0; ok; ++turns) {
+      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_turn[turns & 7]), (turns >> 3) & 1, status, kWaitPReady));
+      if (!ok) break;
+      const uint32_t what = *reinterpret_cast<volatile uint32_t*>(&s_turn[turns & 7]);
+      if (what == 0u) product(std::integral_constant<int, 0>());
+      else if (what == 1u) product(std::integral_constant<int, 1>());
+      else break;
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------- softmax: 64 keys of one query row per thread -------------------------------
+    reg_alloc<104>();
+    const int x = warp >> 3, hf = (warp >> 2) & 1;     // slot, key half (and half of the columns of O in the epilogue)
+    const int row = (warp & 3) * 32 + lane;
+    const int rh = KB == 64 ? (row >> 6) : 0;          // blocks of 64: the tile's query block (whole warps)
+    // A step is one unit of 64 keys per thread, or (blocks of 64) two units, one per key block, of 32 keys per thread: the
+    // unit is what the maximum is taken over, and a row's results must not depend on which block shares a step with it.
+    constexpr int NU = KB == 128 ? 1 : 2, UW = 64 / NU;
+    const int last_key = (KB == 64 ? (row & 63) : row) - UW * hf;   // last key of a unit that the row sees on the diagonal
+    const int pair_bar = 1 + x * 4 + (warp & 3);       // named barrier of the two warps that share these rows
+    const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    const uint32_t tmem_o = tmem + x * 128 + hf * 64 + lane_off, tmem_p = tmem + 384 + x * 64 + hf * (UW / 2) + lane_off;
+    const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
+    float* const xch_mine = &s_xch[x][hf][row];
+    const float* const xch_other = &s_xch[x][hf ^ 1][row];
+    uint32_t n = 0, tiles = 0;
+    // Every warp of the slot passes the barrier at the end of the loop once per tile, and the two warps of a pair meet at
+    // least once per step, also when a wait has given up: `ok` goes through the barriers, so that warps leave the loops
+    // together.
+#pragma unroll 1
+    for (;;) {
+      bool ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_tile[x]), tiles & 1, status, kWaitTmaFull));
+      const DuoTileInfo ti = s_tile[x];
+      const int part_slot = SCHED ? s_part[x] : -1;
+      bool store = false;
+      ++tiles;
+      const bool leave = !ok || (ti.flags & kTileExit);
+      if (!leave) {
+        float m_used = -INFINITY, l_sum = 0.f;   // m_used (of the row) in log2 units of the scaled logits; this half's sum
+        bool first = true;                       // the row has attended nothing yet
+#pragma unroll 1
+        for (bool more = !(ti.flags & kTileEmpty); more; ++n) {
+          ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_s[x]), n & 1, status, kWaitMmaDone));
+          const uint32_t blk = *reinterpret_cast<volatile uint32_t*>(&s_step[x][n & 3]);
+          more = (blk & kStepLast) == 0u;
+          tc_fence_after_sync();
+          uint32_t s[64];
+          {
+            uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
+            uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
+            tmem_ld32(tmem_s + lane_off + hf * UW, s0);
+            tmem_ld32(tmem_s + lane_off + hf * UW + (KB == 128 ? 32 : 64), s1);
+            tmem_wait_ld();
+          }
+          tc_fence_before_sync();
+          __syncwarp();
+          warp_arrive(smem_u32(&bar_sfree));   // S may take the next Q K^T
+          bool any = false;                    // the pair of warps has met in this step
+#pragma unroll
+          for (int u = 0; u < NU; ++u) {
+            // P of the step before has been consumed (its P V runs behind this step's Q K^T)
+            auto wait_p = [&]() {
+              ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady));
+              tc_fence_after_sync();
+            };
+            const uint32_t tp = tmem_p + u * 32;
+            if (KB == 128 || ((blk >> (4 * u + rh)) & 1u)) {     // the row's query block attends the unit's keys
+              if (KB == 128 ? (blk & 1u) : ((blk >> (4 * u + 2 + rh)) & 1u)) {   // diagonal: keys after the query are hidden
+#pragma unroll
+                for (int c = 0; c < UW; ++c)
+                  if (c > last_key) s[u * UW + c] = 0xff800000u;   // -inf
+              }
+              // 2^(s scale - m) to tensor memory as bf16 pairs; returns the sum
+              auto exps = [&]() -> float {
+                const uint64_t negm2 = f2_pack(-m_used, -m_used);
+                uint64_t sum_a = 0ull, sum_b = 0ull;   // (0.f, 0.f)
+#pragma unroll
+                for (int c0 = 0; c0 < UW; c0 += 16) {
+                  uint32_t pk[8];
+#pragma unroll
+                  for (int q = 0; q < 16; q += 4) {
+                    const int c = u * UW + c0 + q;
+                    const uint64_t x01 = f2_fma(f2_pack(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), scale2, negm2);
+                    const uint64_t x23 = f2_fma(f2_pack(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), scale2, negm2);
+                    float x0, x1, x2, x3;
+                    f2_unpack(x01, x0, x1);
+                    f2_unpack(x23, x2, x3);
+                    const float p0 = fast_exp2(x0), p1 = fast_exp2(x1), p2 = fast_exp2(x2), p3 = fast_exp2(x3);
+                    sum_a = f2_add(sum_a, f2_pack(p0, p1));
+                    sum_b = f2_add(sum_b, f2_pack(p2, p3));
+                    pk[q >> 1] = pack_bf16(p0, p1);
+                    pk[(q >> 1) + 1] = pack_bf16(p2, p3);
+                  }
+                  if (c0 == 0) wait_p();
+                  tmem_st8(tp + (c0 >> 1), pk);
+                }
+                float a0, a1, a2, a3;
+                f2_unpack(sum_a, a0, a1);
+                f2_unpack(sum_b, a2, a3);
+                return (a0 + a1) + (a2 + a3);
+              };
+              // Lazy running maximum: the exponentials are first taken against the maximum in use.  Only when a sum shows
+              // that this has gone stale (sum >= kSumLimit, or not finite) is the exact maximum of the row's logits in
+              // the unit taken, O and l rescaled and the unit redone.  A row's first unit has no maximum yet and takes
+              // the exact one straight away.  The maximum is a shift that cancels in O / l: any value that keeps P
+              // finite is right.
+              float hs = 0.f;
+              bool stale = first, redo = true;
+              any = true;
+#pragma unroll 1
+              for (;;) {
+                if (!stale) {
+                  hs = exps();
+                  if (!redo) break;
+                  stale = __any_sync(0xffffffffu, !(hs < kSumLimit));
+                }
+                if (group_all<64>(ok && !stale, pair_bar)) break;
+                ok = group_all<64>(ok, pair_bar);
+                if (!ok) break;
+                float mxa[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) mxa[v] = -INFINITY;
+#pragma unroll
+                for (int c = u * UW; c < u * UW + UW; c += 8) {
+#pragma unroll
+                  for (int v = 0; v < 4; ++v) mxa[v] = max3(mxa[v], __uint_as_float(s[c + 2 * v]), __uint_as_float(s[c + 2 * v + 1]));
+                }
+                const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])) * p.scale_log2;
+                *xch_mine = mx;
+                (void)group_all<64>(true, pair_bar);
+                const float m_new = fmaxf(m_used, fmaxf(mx, *xch_other));
+                const float corr = fast_exp2(m_used - m_new);     // 0 while m_used = -inf
+                l_sum *= corr;
+                m_used = m_new;
+                if (!first) {   // O holds the P V of everything before this unit: rescale this warp's half of its columns
+                  ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady));
+                  tc_fence_after_sync();
+#pragma unroll 1
+                  for (int c0 = 0; c0 < 64; c0 += 16) {
+                    uint32_t r[16];
+                    tmem_ld16(tmem_o + c0, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) * corr);
+                    tmem_st16(tmem_o + c0, r);
+                  }
+                }
+                stale = false;
+                redo = false;
+              }
+              first = false;
+              l_sum += hs;
+            } else {
+              uint32_t zero[8];
+#pragma unroll
+              for (int q = 0; q < 8; ++q) zero[q] = 0u;   // P = 0 for the rows whose block did not select these keys
+              wait_p();
+#pragma unroll
+              for (int c0 = 0; c0 < UW / 2; c0 += 8) tmem_st8(tp + c0, zero);
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            warp_arrive(smem_u32(&bar_in[x][u]));
+          }
+          if (KB == 64 && !any) ok = group_all<64>(ok, pair_bar);
+          if (!ok) break;
+        }
+        // epilogue: O / l -> bf16 -> global
+        const int tok = ti.Tl * 128 + row;
+        const bool in_seq = tok < p.Nq;     // rows of a short last block past the sequence end are not written
+        float* lse_dst = p.lse ? p.lse + (static_cast<int64_t>(ti.l) * p.Hq + ti.h) * p.Nq + tok : nullptr;
+        if (ti.flags & kTileEmpty) {
+          if (in_seq) {
+            __nv_bfloat16* orow = p.O + ti.l * p.osb + static_cast<int64_t>(tok) * p.ost + ti.h * p.osh + hf * 64;
+#pragma unroll 1
+            for (int c = 0; c < 8; ++c) reinterpret_cast<uint4*>(orow)[c] = make_uint4(0, 0, 0, 0);
+            if (lse_dst && hf == 0) *lse_dst = -INFINITY;
+          }
+        } else {
+          ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][NU - 1]), (n - 1) & 1, status, kWaitOReady));
+          tc_fence_after_sync();
+          *xch_mine = l_sum;
+          ok = group_all<64>(ok, pair_bar);
+          l_sum = hf == 0 ? l_sum + *xch_other : *xch_other + l_sum;
+          if (SCHED && part_slot >= 0) {
+            // a part of a split row: the unnormalised O row, the maximum in use and the row sum go to the part's slot;
+            // combine_parts_kernel merges the parts of the row in a fixed order
+            float* po = p.part_o + (static_cast<int64_t>(part_slot) * 128 + row) * 128 + hf * 64;
+#pragma unroll 1
+            for (int c0 = 0; ok && c0 < 64; c0 += 32) {
+              uint32_t r[32];
+              tmem_ld32(tmem_o + c0, r);
+              tmem_wait_ld();
+#pragma unroll
+              for (int q = 0; q < 32; q += 4)
+                *reinterpret_cast<uint4*>(po + c0 + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+            }
+            if (ok && hf == 0) {
+              float* ml = p.part_ml + static_cast<int64_t>(part_slot) * 256;
+              ml[row] = m_used;
+              ml[128 + row] = l_sum;
+            }
+          } else {
+            // into the slot's Q buffer (free since the tile's last Q K^T), in the swizzled layout of a 128-byte-swizzle
+            // tensor map, then two TMA stores: whole 128-byte lines go out, rows past the end of the sequence are clipped
+            const bool empty_row = KB == 64 && !(l_sum > 0.f);   // a row whose own block selected nothing: zeros, lse = -inf
+            const float inv = empty_row ? 0.f : 1.0f / l_sum;
+            const uint32_t srow = smem_u32(sQ) + x * kDuoTile + hf * kDuoPanel + row * 128;
+#pragma unroll 1
+            for (int c0 = 0; ok && c0 < 64; c0 += 32) {
+              uint32_t r[32];
+              tmem_ld32(tmem_o + c0, r);
+              tmem_wait_ld();
+#pragma unroll
+              for (int q = 0; q < 32; q += 8) {
+                uint4 v;
+                v.x = pack_bf16(__uint_as_float(r[q]) * inv, __uint_as_float(r[q + 1]) * inv);
+                v.y = pack_bf16(__uint_as_float(r[q + 2]) * inv, __uint_as_float(r[q + 3]) * inv);
+                v.z = pack_bf16(__uint_as_float(r[q + 4]) * inv, __uint_as_float(r[q + 5]) * inv);
+                v.w = pack_bf16(__uint_as_float(r[q + 6]) * inv, __uint_as_float(r[q + 7]) * inv);
+                if (empty_row) v = make_uint4(0, 0, 0, 0);
+                const uint32_t dst = srow + ((((c0 + q) >> 3) ^ (row & 7)) << 4);   // 16-byte piece of the panel's row
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+              }
+            }
+            store = ok;
+            if (lse_dst && hf == 0 && in_seq && ok && RBS_DBG_OK(tok < p.Nq, status, kDbgPrefillLse))
+              *lse_dst = empty_row ? -INFINITY : (m_used + fast_log2(l_sum)) * 0.6931471805599453f;
+          }
+        }
+        tc_fence_before_sync();
+        fence_proxy_async_smem();
+      }
+      const bool stay = group_all<256>(ok && !leave, 9 + x);   // the slot's eight softmax warps
+      if ((tid & 255) == 0) {
+        if (store && stay) {
+          const uint32_t q_buf = smem_u32(sQ) + x * kDuoTile;
+          tma_store_4d(&tmO, q_buf, 0, ti.h, ti.Tl * 128, ti.l);
+          tma_store_4d(&tmO, q_buf + kDuoPanel, 64, ti.h, ti.Tl * 128, ti.l);
+          tma_store_commit();
+          tma_store_wait_read();
+        }
+        mbar_arrive(smem_u32(&bar_tdone[x]));
+      }
+      if (!stay) break;
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  if (warp == 19) tmem_dealloc(tmem, 512);
+}
+
+// p.band_rows, p.items etc. are set by the caller; n_items: tiles (or items of the schedule), one CTA of the grid each.
+rbs_status launch_prefill_duo(const PrefillParams& p, const rbs_tensor& Q, const rbs_tensor& K, const rbs_tensor& V, int Hkv,
+                              bool blocks64, long long n_items, cudaStream_t s) {
+  CUtensorMap tmQ, tmK, tmV, tmO;
+  rbs_status st;
+  if ((st = make_tmap_lthd(&tmQ, Q.ptr, p.L, p.Nq, p.Hq, kHeadDim, Q.stride_batch, Q.stride_token, Q.stride_head, 64, 128, true)) != RBS_OK) return st;
+  if ((st = make_tmap_lthd(&tmK, K.ptr, p.L, p.N, Hkv, kHeadDim, K.stride_batch, K.stride_token, K.stride_head, 64, blocks64 ? 64 : 128, true)) != RBS_OK) return st;
+  if ((st = make_tmap_panels(&tmV, V.ptr, p.L, p.N, Hkv, V.stride_batch, V.stride_token, V.stride_head, blocks64 ? 64 : 128)) != RBS_OK) return st;
+  if ((st = make_tmap_lthd(&tmO, p.O, p.L, p.Nq, p.Hq, kHeadDim, p.osb, p.ost, p.osh, 64, 128, true)) != RBS_OK) return st;
+  unsigned int* status = device_status_ptr();
+  if (status == nullptr) return RBS_ERR_CUDA;
+  if (n_items > 0x7fffffffLL) return RBS_ERR_UNSUPPORTED;
+  const size_t smem = 2 * kDuoTile + 2 * kDuoStages * kDuoStage;
+  auto launch = [&](auto kern) -> rbs_status {
+    const rbs_status e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
+    if (e != RBS_OK) return e;
+    kern<<<static_cast<unsigned>(n_items), kDuoThreads, smem, s>>>(tmQ, tmK, tmV, tmO, p, status);
+    RBS_CUDA_OK(cudaGetLastError());
+    return RBS_OK;
+  };
+  if (blocks64) return launch(prefill_duo_kernel<64, false>);
+  if (p.items != nullptr) return launch(prefill_duo_kernel<128, true>);
+  return launch(prefill_duo_kernel<128, false>);
+}
+
+}  // namespace rbs

@@ -60,6 +60,22 @@ rbs_status make_tmap_lthd(CUtensorMap* out, const void* ptr, int L, int N, int H
   return r == CUDA_SUCCESS ? RBS_OK : RBS_ERR_CUDA;
 }
 
+// The same tensor viewed as 5-D (j % 64, h, t, l, j / 64): one load brings box_t rows of all 128 columns as two 64-column
+// panels one behind the other (a thread gets a TMA instruction out every 220 cycles, whatever its size).
+rbs_status make_tmap_panels(CUtensorMap* out, const void* ptr, int L, int N, int H, int64_t sb, int64_t st, int64_t sh, int box_t) {
+  EncodeTiledFn fn = encode_fn();
+  if (fn == nullptr) return RBS_ERR_CUDA;
+  cuuint64_t dims[5] = {64, static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(L), kHeadDim / 64};
+  if (sb == 0) sb = st * N;  // batch of one: any valid stride
+  cuuint64_t strides[4] = {static_cast<cuuint64_t>(sh) * 2, static_cast<cuuint64_t>(st) * 2, static_cast<cuuint64_t>(sb) * 2, 128};
+  cuuint32_t box[5] = {64, 1, static_cast<cuuint32_t>(box_t), 1, kHeadDim / 64};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? RBS_OK : RBS_ERR_CUDA;
+}
+
 // Row-major bf16 matrix [rows][cols] (cols contiguous); box = box_cols x box_rows, 128-byte swizzle.
 rbs_status make_tmap_2d(CUtensorMap* out, const void* ptr, int64_t rows, int cols, int box_cols, int box_rows) {
   EncodeTiledFn fn = encode_fn();
