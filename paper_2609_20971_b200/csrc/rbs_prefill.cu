@@ -365,10 +365,17 @@ combine_parts_kernel(const PrefillParams p, const int4* __restrict__ splits) {
   }
 }
 
-// Bands of the tile order: up to four of at least 64 query tiles (512 tiles per band and KV head at G = 8: enough to fill
-// the GPU from one KV head).  Measured at 128K, 32 q / 4 kv heads: 1 / 4 / 8 / 16 bands give 5.52 / 4.86 / 4.97 / 4.90 ms
-// at 3 % density and 17.5 / 16.7 / 17.2 / 17.2 ms at 12 %.
-static int tile_bands(int n_rows) {
+// Bands of the tile order.  Long sequences: up to four of at least 64 query tiles (512 tiles per band and KV head at
+// G = 8: enough to fill the GPU from one KV head).  Measured at 128K, 32 q / 4 kv heads: 1 / 4 / 8 / 16 bands give 5.52 /
+// 4.86 / 4.97 / 4.90 ms at 3 % density and 17.5 / 16.7 / 17.2 / 17.2 ms at 12 %.
+// Where K and V of all heads are small against the 126 MB of L2 nothing is gained by taking the KV heads one after the
+// other, and the last one's long rows would start late and end alone (8K tokens, 32 q / 4 kv heads: the last CTA ended
+// after 213 us, the median after 172): as many bands as rows, i.e. longest rows first over all heads.  Launched back to
+// back, bands against rows: 8K (16 MiB of K and V) 233 / 209 us, 16K with 8 kv heads (64 MiB) 648 / 647, 32K (64 MiB) 1417 /
+// 1438, 64K (128 MiB) 3017 / 3183.
+constexpr double kRowOrderBytes = 40.0 * 1024 * 1024;
+static int tile_bands(int n_rows, bool scheduled, double kv_bytes) {
+  if (!scheduled && kv_bytes <= kRowOrderBytes) return n_rows;
   const int n_bands = n_rows / 64;
   return n_bands < 1 ? 1 : (n_bands > 4 ? 4 : n_bands);
 }
@@ -378,16 +385,19 @@ static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q,
   rbs_status st;
   PrefillParams pp = p;
   const int n_rows = p.Mq * p.R;
-  const int n_bands = tile_bands(n_rows);
+  // the schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink
+  // steadily) and a group whose counts fit the planner's shared memory
+  const double kv_bytes = 4.0 * kHeadDim * p.L * Hkv * static_cast<double>(p.N);
+  const int sched_bands = tile_bands(n_rows, true, 0.0);
+  const bool scheduled = p.mask != nullptr && workspace != nullptr &&
+                         static_cast<size_t>((n_rows + sched_bands - 1) / sched_bands) * p.G * sizeof(int) <= 200 * 1024;
+  const int n_bands = tile_bands(n_rows, scheduled, kv_bytes);
   pp.band_rows = (n_rows + n_bands - 1) / n_bands;
   const int n_groups = n_bands * p.L * Hkv;
   const int rows_per_group = pp.band_rows * p.G;
   pp.items = nullptr; pp.items_per_group = 0; pp.part_o = nullptr; pp.part_ml = nullptr;
   int4* splits = nullptr;
-  // the schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink
-  // steadily) and a group whose counts fit the planner's shared memory
   const size_t plan_smem = static_cast<size_t>(rows_per_group) * sizeof(int);
-  const bool scheduled = p.mask != nullptr && workspace != nullptr && plan_smem <= 200 * 1024;
   if (scheduled) {
     const PrefillWorkspace w = prefill_workspace(p.L, p.Hq, Hkv, p.M * p.R, p.G);
     if (workspace_bytes < w.bytes || reinterpret_cast<uintptr_t>(workspace) % 256 != 0) return RBS_ERR_WORKSPACE;
@@ -416,7 +426,7 @@ static rbs_status launch_prefill_tc64(const PrefillParams& p, const rbs_tensor& 
                                       const rbs_tensor& V, int Hkv, cudaStream_t s) {
   PrefillParams pp = p;
   const int n_rows = (p.Mq + 1) / 2;
-  const int n_bands = tile_bands(n_rows);
+  const int n_bands = tile_bands(n_rows, false, 4.0 * kHeadDim * p.L * Hkv * static_cast<double>(p.N));
   pp.band_rows = (n_rows + n_bands - 1) / n_bands;
   return launch_prefill_duo(pp, Q, K, V, Hkv, true, static_cast<long long>(p.L) * p.Hq * pp.band_rows * n_bands, s);
 }

@@ -41,7 +41,8 @@ constexpr uint32_t kDuoTile = 2 * kDuoPanel;  // one Q tile
 // Blocks of 128 and more: bit 0: the step's keys are the tile's diagonal sub-block.  Blocks of 64: bits 0-3 describe the
 // step's first key block, bits 4-7 its second (bit 0 / 1: selected by query block A / B of the tile, bit 2 / 3: it is
 // the diagonal block of A / B).
-enum : uint32_t { kStepLast = 1u << 8, kStepOneHalf = 1u << 9, kStepExit = 1u << 31 };
+// kStepTileParity: of the number of tiles announced before this one.
+enum : uint32_t { kStepLast = 1u << 8, kStepOneHalf = 1u << 9, kStepTileParity = 1u << 10, kStepExit = 1u << 31 };
 enum : int { kTileExit = 1, kTileEmpty = 2 };
 struct DuoTileInfo { int Tl, h, l, flags; };
 
@@ -99,19 +100,66 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 // Walks the steps of one tile.  KB = 128: every step is one selected 128-key sub-block of the tile's mask row.
 // KB = 64: the tile holds two consecutive query blocks of 64 (rows 0-63: block iA, rows 64-127: iB = iA + 1), each with
 // its own mask row; a step is two consecutive key blocks of the UNION of the two rows.
+// The rest of the current mask word is kept in a register and the next word is on its way: with a walk that read the
+// mask anew for every step a producer spent 700 - 950 cycles of a step on it.
 template <int KB>
 struct StepWalk;
 
+// the bits of word w that belong to blocks <= last
+__device__ __forceinline__ uint32_t causal_bits(int w, int last) {
+  const int n = last - (w << 5);
+  return n >= 31 ? 0xffffffffu : n < 0 ? 0u : 0xffffffffu >> (31 - n);
+}
+
 template <>
 struct StepWalk<128> {
-  const uint32_t* row; int i, R, T, Tw, cur;
-  __device__ __forceinline__ void start(int kb0) { cur = next_kb(row, kb0, i, R, Tw); }
+  const uint32_t* row;        // null: dense
+  int i, T, Tw, cur;          // query block, tile, last sub-block this walk may take, current sub-block (-1: none)
+  int w; uint32_t u, ahead;   // word, its blocks still to come, the next word
+  bool two;                   // blocks of 256: two sub-blocks each
+  __device__ __forceinline__ void load(int w0) {
+    w = w0;
+    ahead = w0 <= (i >> 5) ? __ldg(row + w0) : 0u;
+  }
+  __device__ __forceinline__ void next() {
+    if (row == nullptr) {
+      cur = cur < Tw ? cur + 1 : -1;
+      return;
+    }
+    if (two && cur >= 0 && !(cur & 1)) {        // the second sub-block of the same block
+      cur = cur < Tw ? cur + 1 : -1;
+      return;
+    }
+    while (u == 0u) {
+      if (w > (i >> 5)) { cur = -1; return; }
+      u = ahead & causal_bits(w, i);
+      load(w + 1);
+    }
+    const int b = ((w - 1) << 5) + __ffs(u) - 1;
+    u &= u - 1u;
+    cur = two ? 2 * b : b;
+    if (cur > Tw) cur = -1;
+  }
+  __device__ __forceinline__ void start(int kb0, int R) {     // kb0: the sub-block in front of the first one
+    two = R == 2;
+    if (row == nullptr) { cur = kb0; next(); return; }
+    const int kb = kb0 + 1, b = two ? kb >> 1 : kb;
+    load(b >> 5);
+    u = 0u;
+    cur = -1;
+    if (w <= (i >> 5)) {
+      u = ahead & causal_bits(w, i) & (0xffffffffu << (b & 31));
+      load(w + 1);
+    }
+    next();
+    if (two && (kb & 1) && cur == kb - 1) next();             // a part that starts in the middle of a block
+  }
   __device__ __forceinline__ bool any() const { return cur >= 0; }
   // the current step: first key row of its two halves of 64 keys, flags; then moves on
   __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
     r0 = cur * 128; r1 = r0 + 64;
     uint32_t f = cur == T ? 1u : 0u;
-    cur = next_kb(row, cur, i, R, Tw);
+    next();
     if (cur < 0) f |= kStepLast;
     return f;
   }
@@ -121,42 +169,36 @@ template <>
 struct StepWalk<64> {
   const uint32_t* rowA; const uint32_t* rowB;   // mask rows of the two query blocks (rowB null: no second block)
   int iA, iB, cur;
-  __device__ __forceinline__ int next(int from) const {   // next key block after `from` selected by either row, or -1
-    const int last = rowB ? iB : iA;
-    int b = from + 1;
-    while (b <= last) {
-      const int w = b >> 5;
-      uint32_t u = __ldg(rowA + w);
-      if (((w + 1) << 5) - 1 > iA) u = (w << 5) > iA ? 0u : (u & (0xffffffffu >> (31 - (iA & 31))));
-      if (rowB) {
-        uint32_t v = __ldg(rowB + w);
-        if (((w + 1) << 5) - 1 > iB) v = (w << 5) > iB ? 0u : (v & (0xffffffffu >> (31 - (iB & 31))));
-        u |= v;
-      }
-      u >>= (b & 31);
-      if (u) return b + __ffs(u) - 1;
-      b = (b | 31) + 1;
+  int w; uint32_t ua, ub, aheadA, aheadB;       // word, the rows' blocks still to come in it, the next words
+  uint32_t f_cur;                               // flags of the current block (see kStepLast above)
+  __device__ __forceinline__ void load(int w0) {
+    w = w0;
+    aheadA = w0 <= (iA >> 5) ? __ldg(rowA + w0) : 0u;
+    aheadB = rowB && w0 <= (iB >> 5) ? __ldg(rowB + w0) : 0u;
+  }
+  __device__ __forceinline__ void next() {
+    while ((ua | ub) == 0u) {
+      if (w > (iB >> 5)) { cur = -1; return; }
+      ua = aheadA & causal_bits(w, iA);
+      ub = aheadB & causal_bits(w, iB);
+      load(w + 1);
     }
-    return -1;
+    const uint32_t low = (ua | ub) & (0u - (ua | ub));
+    cur = ((w - 1) << 5) + __ffs(low) - 1;
+    f_cur = ((ua & low) ? 1u : 0u) | ((ub & low) ? 2u : 0u) | (cur == iA ? 4u : 0u) | (cur == iB ? 8u : 0u);
+    ua &= ~low;
+    ub &= ~low;
   }
-  __device__ __forceinline__ uint32_t flags(int b) const {
-    uint32_t f = 0;
-    if (b <= iA && ((__ldg(rowA + (b >> 5)) >> (b & 31)) & 1u)) f |= 1u;
-    if (rowB && b <= iB && ((__ldg(rowB + (b >> 5)) >> (b & 31)) & 1u)) f |= 2u;
-    if (b == iA) f |= 4u;
-    if (b == iB) f |= 8u;
-    return f;
-  }
-  __device__ __forceinline__ void start(int) { cur = next(-1); }
+  __device__ __forceinline__ void start(int, int) { load(0); ua = ub = 0u; next(); }
   __device__ __forceinline__ bool any() const { return cur >= 0; }
   __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
     r0 = cur * 64;
-    uint32_t f = flags(cur);
-    const int b1 = next(cur);
-    if (b1 < 0) { cur = -1; return f | kStepLast | kStepOneHalf; }
-    r1 = b1 * 64;
-    f |= flags(b1) << 4;
-    cur = next(b1);
+    uint32_t f = f_cur;
+    next();
+    if (cur < 0) return f | kStepLast | kStepOneHalf;
+    r1 = cur * 64;
+    f |= f_cur << 4;
+    next();
     if (cur < 0) f |= kStepLast;
     return f;
   }
@@ -173,17 +215,18 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sQ = smem;                    // [slot][kDuoTile]
   unsigned char* sKV = smem + 2 * kDuoTile;    // [slot][kDuoStages][kDuoStage]
-  __shared__ __align__(16) uint32_t s_clc[4];
+  __shared__ __align__(16) uint32_t s_clc[2][4];
   // per slot.  k: the K of an even / odd step is there; in: P and V are there (eight softmax warps and the producer
-  // arrive); s: S is there, K is free; pv: P V is done, P and V are free (in, pv: with blocks of 64 one per key block); tile / tdone: a tile has been announced / its
-  // output is out.  sfree: S has been read into registers; turn: messages of warp 18 to warp 19
+  // arrive); s: S is there, K is free; pv: P V is done, P and V are free (in, pv: with blocks of 64 one per key block);
+  // tile: an even / odd tile has been announced; tdone: its O has been read; ofree: its output has left the V buffer.
+  // sfree: S has been read into registers; turn: messages of warp 18 to warp 19
   __shared__ __align__(8) uint64_t bar_k[2][2], bar_in[2][2], bar_s[2], bar_pv[2][2], bar_sfree, bar_turn[8];
-  __shared__ __align__(8) uint64_t bar_q[2], bar_tile[2], bar_tdone[2], bar_clc;
+  __shared__ __align__(8) uint64_t bar_q[2], bar_tile[2][2], bar_tdone[2], bar_ofree[2], bar_clc[2];
   __shared__ float s_xch[2][2][128];             // [slot][key half][row]: maxima, row sums for the other key half
   __shared__ uint32_t s_step[2][4], s_turn[8];   // turn: the slot whose P V is due
-  __shared__ DuoTileInfo s_tile[2];
-  __shared__ int s_part[2];
-  __shared__ uint32_t s_tmem, s_lock, s_clc_phase, s_no_more;
+  __shared__ DuoTileInfo s_tile[2][2];           // [slot][tile parity]
+  __shared__ int s_part[2][2];
+  __shared__ uint32_t s_tmem, s_lock, s_no_more;
 
   const int tid = threadIdx.x, lane = tid & 31;
   // uniform for the compiler: the roles then run on uniform registers and branches (20 % less code, 55 instead of 128 moves
@@ -194,15 +237,16 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     for (int x = 0; x < 2; ++x) {
       for (int k = 0; k < 2; ++k) {
         mbar_init(smem_u32(&bar_k[x][k]), 2);
+        mbar_init(smem_u32(&bar_tile[x][k]), 1);
         mbar_init(smem_u32(&bar_in[x][k]), 9); mbar_init(smem_u32(&bar_pv[x][k]), 1);
       }
       mbar_init(smem_u32(&bar_s[x]), 1); 
-      mbar_init(smem_u32(&bar_q[x]), 1); mbar_init(smem_u32(&bar_tile[x]), 1); mbar_init(smem_u32(&bar_tdone[x]), 1);
+      mbar_init(smem_u32(&bar_q[x]), 1); mbar_init(smem_u32(&bar_tdone[x]), 1); mbar_init(smem_u32(&bar_ofree[x]), 1);
+      mbar_init(smem_u32(&bar_clc[x]), 1);
     }
     for (int k = 0; k < 8; ++k) mbar_init(smem_u32(&bar_turn[k]), 1);
     mbar_init(smem_u32(&bar_sfree), 8);
-    mbar_init(smem_u32(&bar_clc), 1);
-    s_lock = 0; s_clc_phase = 0; s_no_more = 0;
+    s_lock = 0; s_no_more = 0;
     mbar_fence_init();
   }
   if (warp == 19) tmem_alloc(smem_u32(&s_tmem), 512);
@@ -219,44 +263,52 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     if (lane == 0) {
       const int x = warp - 16;
       if (x == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmO); } else { tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); }
-      // the next tile of the grid, or -1: two threads of the CTA share one request at a time; a request that finds no
-      // CTA left to cancel is the last one made
-      auto fetch = [&]() -> int {
-        bool locked = false;
+      // Asks for the next tile of the grid / takes the answer (-1: none is left).  The two producers ask independently,
+      // but none asks once a request is known to have found no CTA left to cancel: the lock covers asking and looking.
+      uint32_t asked = 0;
+      bool pending = false;
+      const uint32_t resp = smem_u32(s_clc[x]), clc_bar = smem_u32(&bar_clc[x]);
+      auto lock = [&]() -> bool {
 #pragma unroll 1
         for (uint32_t it = 0; it < kSpinLimit; ++it) {
-          if (atomicCAS(&s_lock, 0u, 1u) == 0u) { locked = true; break; }
+          if (atomicCAS(&s_lock, 0u, 1u) == 0u) { __threadfence_block(); return true; }
           if (it > 64) __nanosleep(64);
           if ((it & 255u) == 255u && *reinterpret_cast<volatile unsigned int*>(status) != 0u) break;
         }
-        if (!locked) { atomicCAS(status, 0u, static_cast<unsigned int>(kWaitStageFree)); return -1; }
-        __threadfence_block();
-        int got = -1;
+        atomicCAS(status, 0u, static_cast<unsigned int>(kWaitStageFree));
+        return false;
+      };
+      auto unlock = [&]() { __threadfence_block(); atomicExch(&s_lock, 0u); };
+      auto ask = [&]() {
+        pending = false;
+        if (!lock()) return;
         if (*reinterpret_cast<volatile uint32_t*>(&s_no_more) == 0u) {
-          const uint32_t ph = *reinterpret_cast<volatile uint32_t*>(&s_clc_phase);
-          const uint32_t resp = smem_u32(s_clc), bar = smem_u32(&bar_clc);
           fence_proxy_async_smem();                 // the last response has been read
-          mbar_arrive_expect_tx(bar, 16);
+          mbar_arrive_expect_tx(clc_bar, 16);
           asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
-                       ::"r"(resp), "r"(bar) : "memory");
-          uint32_t ok = 0, cx = 0;
-          if (duo_wait(bar, ph, status, kWaitTmaFull)) {
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
-                "ld.shared.b128 r, [%2];\n\t"
-                "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t"
-                "mov.u32 %1, 0;\n\t"
-                "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n\t}"
-                : "=r"(ok), "=r"(cx) : "r"(resp) : "memory");
-          }
-          if (ok) got = static_cast<int>(cx);
-          else s_no_more = 1u;
-          s_clc_phase = ph ^ 1u;
+                       ::"r"(resp), "r"(clc_bar) : "memory");
+          pending = true;
         }
-        __threadfence_block();
-        atomicExch(&s_lock, 0u);
-        return got;
+        unlock();
+      };
+      auto answer = [&]() -> int {
+        if (!pending) return -1;
+        pending = false;
+        if (!duo_wait(clc_bar, asked & 1, status, kWaitTmaFull)) return -1;
+        ++asked;
+        if (!lock()) return -1;
+        uint32_t got, cx;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+            "ld.shared.b128 r, [%2];\n\t"
+            "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t"
+            "mov.u32 %1, 0;\n\t"
+            "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n\t}"
+            : "=r"(got), "=r"(cx) : "r"(resp) : "memory");
+        if (!got) s_no_more = 1u;
+        unlock();
+        return got ? static_cast<int>(cx) : -1;
       };
       const uint64_t pol_q = make_policy_evict_first();
       const uint32_t q_dst = smem_u32(sQ) + x * kDuoTile, kv_dst = smem_u32(sKV) + x * kDuoStages * kDuoStage;
@@ -306,82 +358,100 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int per_band_kv = SCHED ? p.items_per_group : p.band_rows * p.G;
       const int per_band = p.L * Hkv * per_band_kv;
       const int n_rows = KB == 128 ? p.Mq * p.R : (p.Mq + 1) / 2;    // 128-row tiles of the call
-      // -2: to be fetched; a launch in which a wait has given up is lost: CTAs that start after that do nothing
-      int w = *reinterpret_cast<volatile unsigned int*>(status) != 0u ? -1 : x == 0 ? static_cast<int>(blockIdx.x) : -2;
+      int w = static_cast<int>(blockIdx.x);       // slot A's first tile; every other one is asked for
+      if (x != 0) { ask(); w = answer(); }
+      // a launch in which a wait has given up is lost: CTAs that start after that do nothing (looked at after the first
+      // tile's mask has been requested, so that the two latencies pass together)
+      uint32_t lost = *reinterpret_cast<volatile unsigned int*>(status);
 #pragma unroll 1
-      while (ok) {
-        if (w == -2) w = fetch();
-        if (w < 0) break;
+      while (ok && w >= 0) {
         // Tile order: the query tiles are cut into bands of band_rows consecutive tiles, the last (longest) band first;
         // inside a band one (batch, KV head) at a time, inside it longest rows first, the G query heads of the group
         // together.  All tiles in flight then read the K/V of one KV head (64 MiB at 128K tokens), which stays in L2;
         // with all KV heads interleaved the K/V tiles of a 128K layer (256 MiB) were re-read from DRAM many times.
         // The bands keep the very long rows (the dense rows of the last query blocks) of every KV head near the start
-        // of the launch.  SCHED: the item list of plan_rows_kernel instead: the same order, long rows cut into parts.
+        // of the launch.  Where K and V of all heads fit L2 together there are as many bands as rows: longest rows first
+        // over all heads.  SCHED: the item list of plan_rows_kernel instead: the same order, long rows cut into parts.
         const int band = w / per_band, rem_band = w % per_band;
         const int kvid = rem_band / per_band_kv;
         int rem = rem_band % per_band_kv;
         int4 item = make_int4(0, 0, 0x7fffffff, -1);
         if (SCHED) { item = __ldg(p.items + w); rem = item.x; }
-        w = -2;
         const int l = kvid / Hkv, hk = kvid % Hkv;
         const int Tl = n_rows - 1 - (band * p.band_rows + rem / p.G);
-        if ((SCHED && item.x < 0) || Tl < 0 || Tl * 128 >= p.Nq) continue;   // no such tile
+        if ((SCHED && item.x < 0) || Tl < 0 || Tl * 128 >= p.Nq) {    // no such tile
+          ask();
+          w = answer();
+          continue;
+        }
         const int h = hk * p.G + rem % p.G;
+        // Q is on its way to L2 while the mask is read
+        tma_prefetch_4d(&tmQ, 0, h, Tl * 128, l);
+        tma_prefetch_4d(&tmQ, 64, h, Tl * 128, l);
         StepWalk<KB> walk;
         if constexpr (KB == 128) {
           const int T = p.q0 * p.R + Tl, i = T / p.R;
           if (!RBS_DBG_OK(i >= p.q0 && i - p.q0 < p.Mq && h < p.Hq && l < p.L && T < p.M * p.R, status, kDbgPrefillTile)) break;
           walk.row = p.mask ? p.mask + ((static_cast<int64_t>(l) * p.Hq + h - rem % p.G % p.mask_heads) * p.Mq + (i - p.q0)) * p.W : nullptr;
-          walk.i = i; walk.R = p.R; walk.T = T;
+          walk.i = i; walk.T = T;
           walk.Tw = SCHED ? min(T, item.z - 1) : T;
-          walk.start(SCHED ? item.y - 1 : -1);
+          walk.start(SCHED ? item.y - 1 : -1, p.R);
         } else {
           walk.iA = p.q0 + 2 * Tl; walk.iB = walk.iA + 1;
           walk.rowA = p.mask + ((static_cast<int64_t>(l) * p.Hq + h) * p.Mq + 2 * Tl) * p.W;
           walk.rowB = (2 * Tl + 1 < p.Mq) ? walk.rowA + p.W : nullptr;
-          walk.start(-1);
+          walk.start(-1, 0);
         }
         const bool empty = !walk.any();
+        if (lost != 0u) break;
         int r0 = 0, r1 = 0, v0 = 0, v1 = 0;
         uint32_t info = 0, vinfo = 0;
+        bool first_v = true;
 #pragma unroll 1
         for (bool begin = true;; begin = false) {   // the K of a step in front of the V of the step before it
           if (begin ? !empty : !(vinfo & kStepLast)) {
             info = walk.take(r0, r1);
             if (!RBS_DBG_OK(r0 < p.N, status, kDbgPrefillBlock)) { ok = false; break; }
-            load_k(r0, r1, info, hk, l);
+            load_k(r0, r1, begin ? info | ((pub & 1) ? kStepTileParity : 0u) : info, hk, l);
+            // the next tile is asked for with the last K: the answer is there when this tile's last V is out (asked for
+            // earlier, the tiles of a small grid would pile up at the first CTAs to ask)
+            if (info & kStepLast) ask();
           }
           if (begin) {
-            // the slot's Q buffer (also the staging buffer of its output) and tile record are free once its last tile is done
-            if (ok) ok = duo_wait(smem_u32(&bar_tdone[x]), (pub - 1) & 1, status, kWaitStageFree);
+            // A tile is announced, and its Q requested, while the one before it is under way: Q is free since that one's
+            // last Q K^T (the wait for K panel 1).  The tile before that is done: its ofree has been waited for, with the
+            // first V of the tile before this one, or here.
+            if (empty) ok = duo_wait(smem_u32(&bar_ofree[x]), (pub - 1) & 1, status, kWaitStageFree);
             if (!ok) break;
-            s_tile[x].Tl = Tl; s_tile[x].h = h; s_tile[x].l = l; s_tile[x].flags = empty ? kTileEmpty : 0;
-            if (SCHED) s_part[x] = item.w;
-            mbar_arrive(smem_u32(&bar_tile[x]));
+            s_tile[x][pub & 1] = DuoTileInfo{Tl, h, l, empty ? kTileEmpty : 0};
+            if (SCHED) s_part[x][pub & 1] = item.w;
+            mbar_arrive(smem_u32(&bar_tile[x][pub & 1]));
             ++pub;
-            if (empty) break;
+            if (empty) { ask(); break; }
             // Q is read exactly once per launch: evict-first, so that it does not push the K/V in flight out of L2
             mbar_arrive_expect_tx(smem_u32(&bar_q[x]), kDuoTile);
             tma_load_4d_hint(q_dst, &tmQ, smem_u32(&bar_q[x]), 0, h, Tl * 128, l, pol_q);
             tma_load_4d_hint(q_dst + kDuoPanel, &tmQ, smem_u32(&bar_q[x]), 64, h, Tl * 128, l, pol_q);
           } else if (ok) {
-            load_v(v0, v1, vinfo, hk, l);
+            if (first_v) {     // the V buffer takes the output of the tile before
+              ok = duo_wait(smem_u32(&bar_ofree[x]), pub & 1, status, kWaitStageFree);
+              first_v = false;
+            }
+            if (ok) load_v(v0, v1, vinfo, hk, l);
           }
           if (!ok || (!begin && (vinfo & kStepLast))) break;
           v0 = r0; v1 = r1; vinfo = info;
         }
+        w = ok ? answer() : -1;
       }
+      if (pending) (void)answer();     // (after a failure: the response must not arrive behind the CTA's end)
       // no tile left: the issuer learns it from a step, the softmax warps from a tile
       if (ok) {
         s_step[x][nk & 3] = kStepExit;
         mbar_arrive(smem_u32(&bar_k[x][nk & 1]));
         mbar_arrive(smem_u32(&bar_k[x][nk & 1]));
-        ok = duo_wait(smem_u32(&bar_tdone[x]), (pub - 1) & 1, status, kWaitStageFree);
-        if (ok) {
-          s_tile[x].flags = kTileExit;
-          mbar_arrive(smem_u32(&bar_tile[x]));
-        }
+        s_tile[x][pub & 1].flags = kTileExit;
+        mbar_arrive(smem_u32(&bar_tile[x][pub & 1]));
       }
     }
     __syncwarp();
@@ -421,7 +491,9 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const uint32_t info = *reinterpret_cast<volatile uint32_t*>(&s_step[X][n[X] & 3]);
       if (!mid[X]) {
         if (info & kStepExit) { done[X] = true; return true; }
-        if (!__all_sync(0xffffffffu, mbar_test(smem_u32(&bar_q[X]), tiles[X] & 1))) return false;
+        // Q is there, and the softmax warps are done with the slot's last tile (else they would keep S from the other slot)
+        if (!__all_sync(0xffffffffu, mbar_test(smem_u32(&bar_q[X]), tiles[X] & 1) &&
+                                         mbar_test(smem_u32(&bar_tdone[X]), (info & kStepTileParity) ? 0u : 1u))) return false;
         ++tiles[X];
       }
       ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_sfree), (uses - 1) & 1, status, kWaitTmemFree));
@@ -511,9 +583,9 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     // together.
 #pragma unroll 1
     for (;;) {
-      bool ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_tile[x]), tiles & 1, status, kWaitTmaFull));
-      const DuoTileInfo ti = s_tile[x];
-      const int part_slot = SCHED ? s_part[x] : -1;
+      bool ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_tile[x][tiles & 1]), (tiles >> 1) & 1, status, kWaitTmaFull));
+      const DuoTileInfo ti = s_tile[x][tiles & 1];
+      const int part_slot = SCHED ? s_part[x][tiles & 1] : -1;
       bool store = false;
       ++tiles;
       const bool leave = !ok || (ti.flags & kTileExit);
@@ -684,11 +756,11 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
               ml[128 + row] = l_sum;
             }
           } else {
-            // into the slot's Q buffer (free since the tile's last Q K^T), in the swizzled layout of a 128-byte-swizzle
+            // into the slot's V buffer (free since the tile's last P V), in the swizzled layout of a 128-byte-swizzle
             // tensor map, then two TMA stores: whole 128-byte lines go out, rows past the end of the sequence are clipped
             const bool empty_row = KB == 64 && !(l_sum > 0.f);   // a row whose own block selected nothing: zeros, lse = -inf
             const float inv = empty_row ? 0.f : 1.0f / l_sum;
-            const uint32_t srow = smem_u32(sQ) + x * kDuoTile + hf * kDuoPanel + row * 128;
+            const uint32_t srow = smem_u32(sKV) + (x * kDuoStages + 3) * kDuoStage + hf * kDuoPanel + row * 128;
 #pragma unroll 1
             for (int c0 = 0; ok && c0 < 64; c0 += 32) {
               uint32_t r[32];
@@ -717,13 +789,14 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const bool stay = group_all<256>(ok && !leave, 9 + x);   // the slot's eight softmax warps
       if ((tid & 255) == 0) {
         if (store && stay) {
-          const uint32_t q_buf = smem_u32(sQ) + x * kDuoTile;
-          tma_store_4d(&tmO, q_buf, 0, ti.h, ti.Tl * 128, ti.l);
-          tma_store_4d(&tmO, q_buf + kDuoPanel, 64, ti.h, ti.Tl * 128, ti.l);
+          const uint32_t o_buf = smem_u32(sKV) + (x * kDuoStages + 3) * kDuoStage;
+          tma_store_4d(&tmO, o_buf, 0, ti.h, ti.Tl * 128, ti.l);
+          tma_store_4d(&tmO, o_buf + kDuoPanel, 64, ti.h, ti.Tl * 128, ti.l);
           tma_store_commit();
-          tma_store_wait_read();
         }
         mbar_arrive(smem_u32(&bar_tdone[x]));
+        if (store && stay) tma_store_wait_read();
+        mbar_arrive(smem_u32(&bar_ofree[x]));
       }
       if (!stay) break;
     }
