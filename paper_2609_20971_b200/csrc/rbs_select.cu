@@ -177,7 +177,8 @@ select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   __shared__ __align__(8) uint64_t bar_q, bar_cfull[2], bar_cempty[2], bar_tfull[2], bar_tempty[2];   // c*: [0] hi half, [1] lo half
   __shared__ uint32_t s_tmem;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform for the compiler, see select_pair_kernel
   const int per_i = p.L * p.Hq;
   const int il = p.Mq - 1 - static_cast<int>(blockIdx.x / per_i);   // query block inside this call's chunk
   const int i = p.q0 + il;                                            // its position in the sequence
@@ -363,7 +364,11 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __shared__ float sRed[2][2][8], sRedQ[2][16], sQstat[2][2];
   __shared__ uint32_t s_tmem;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // The warp index from a shuffle is uniform for the compiler, so that the roles run on uniform branches and registers
+  // instead of moving every MMA operand there: 1.57 against 1.65 ms on the 128K layer of 32 heads, 6.66 against 7.33 ms on
+  // the 64-head layer at blocks of 64, 0.70 against 0.77 ms at 64K.
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int Hkv = p.Hq / p.G, GP = HALVES ? p.G : p.G / 2;   // items per (batch, KV head, query block)
   const int per_i = p.L * Hkv * GP;
   constexpr int QB = HALVES ? 2 * B : B;                     // tokens of a query block
