@@ -36,8 +36,8 @@ NCU_TRAFFIC_BYTES = {
 NOMINAL_BF16_TFLOPS = 2250.0     # dense bf16 per B200, for context next to the measured peak
 TARGET_TENSOR_FRAC = 0.60        # select + sparse attention on the selected FLOPs, of the measured bf16 peak
 TARGET_HBM_FRAC = 0.70           # statistics pass, of the measured copy bandwidth
-# kernels per step of the path: block_stats; rescue_coeff, split_centroid, select_pair, density; prefill_duo
-LAUNCHES_PER_STEP = 6
+# kernels per step of the path: block_stats; select_prep, select_pair; prefill_duo
+LAUNCHES_PER_STEP = 4
 # the bounded oracle sample both arms time (the same in `cpu_baseline` and in `--impl reference`)
 ORACLE_SAMPLE = dict(n_heads=4, n_att_rows=48)
 

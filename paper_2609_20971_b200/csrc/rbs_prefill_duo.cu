@@ -253,6 +253,8 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = s_tmem;
   const uint32_t tmem_s = tmem + 256;
   const int Hkv = p.Hq / p.G;
@@ -823,8 +825,7 @@ rbs_status launch_prefill_duo(const PrefillParams& p, const rbs_tensor& Q, const
   auto launch = [&](auto kern) -> rbs_status {
     const rbs_status e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != RBS_OK) return e;
-    kern<<<static_cast<unsigned>(n_items), kDuoThreads, smem, s>>>(tmQ, tmK, tmV, tmO, p, status);
-    RBS_CUDA_OK(cudaGetLastError());
+    RBS_CUDA_OK(launch_pdl(kern, static_cast<unsigned>(n_items), 1, kDuoThreads, smem, s, tmQ, tmK, tmV, tmO, p, status));
     return RBS_OK;
   };
   if (blocks64) return launch(prefill_duo_kernel<64, false>);

@@ -14,29 +14,45 @@
 namespace rbs {
 
 // ---------------------------------------------------------------------------------------------
-// 1. per (l, KV head): sort radii, quantiles, beta, g = r * beta
+// 1. per (l, KV head): sort radii, quantiles, beta, g = r * beta; fp32 centroid -> bf16 hi + bf16 lo, rows padded to Mpad
+//    with zeros
 // ---------------------------------------------------------------------------------------------
-constexpr int kCoeffThreads = 1024;
+constexpr int kPrepThreads = 1024;
 
 // Besides beta, the kernel fixes the ORDER in which the scoring kernels see the blocks of each 128-row centroid tile:
 // inside a tile the rows with r_b beta_b = 0 (at least half of all blocks: every radius at or below the median) come
 // first, the others after them (the other way round in odd tiles).  perm[pos] = block index, gs[pos] = r_b beta_b scale
 // (log2 units per unit of query norm) in that order.  A scoring warp whose 32 rows all have gs = 0 then needs no
 // second exponential per logit, because S_rescue = S_base there; without the partition hardly any warp would qualify.
-__global__ void __launch_bounds__(kCoeffThreads)
-rescue_coeff_kernel(const float* __restrict__ radius, int M, int P /* pow2 >= M */, float scale_log2,
-                    float* __restrict__ beta, float* __restrict__ rq, float* __restrict__ gs, int* __restrict__ perm,
-                    int Mpad, int beta_mode /* 0: Eq. (beta), 1: beta = 0, 2: beta = 1 */) {
+// The split copies of the centroids are multiplied by log2(e)/sqrt(d), so that the tensor-core product is the scaled logit
+// in log2 units; cnorm is the norm of the scaled centroid.
+// One CTA per (l, KV head) and slice of the centroid tiles: every slice sorts the radii again, which costs less than the
+// launch that would share one sort; the counters of the scoring kernel are cleared here for the same reason (three
+// launches, a memset among them, in one).
+__global__ void __launch_bounds__(kPrepThreads)
+select_prep_kernel(const float* __restrict__ radius, const float* __restrict__ centroid, int M, int P /* pow2 >= M */,
+                   float scale_log2, float* __restrict__ beta, float* __restrict__ rq, float* __restrict__ gs,
+                   int* __restrict__ perm, __nv_bfloat16* __restrict__ chi, __nv_bfloat16* __restrict__ clo,
+                   float* __restrict__ cnorm, int Mpad, int tiles_per_slice,
+                   int beta_mode /* 0: Eq. (beta), 1: beta = 0, 2: beta = 1 */, unsigned int* __restrict__ counts, int n_counts,
+                   unsigned int* __restrict__ done) {
   extern __shared__ float s_sorted[];
   __shared__ float s_q[2];
-  __shared__ unsigned short s_zero[8192 / 32];   // per group of 32 rows: how many have gs = 0
-  const int hd = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  __shared__ unsigned short s_zero[kPrepThreads / 32];   // per group of 32 rows: how many have gs = 0
+  __shared__ int s_dst[kPrepThreads];                    // where a row of the group goes
+  const int hd = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  pdl_trigger();
+  if (blockIdx.y == 0) {
+    for (int k = hd * kPrepThreads + tid; k < n_counts; k += gridDim.x * kPrepThreads) counts[k] = 0u;
+    if (hd == 0 && tid == 0) *done = 0u;
+  }
   const float* r = radius + static_cast<int64_t>(hd) * M;
-  for (int idx = tid; idx < P; idx += kCoeffThreads) s_sorted[idx] = idx < M ? r[idx] : __int_as_float(0x7f800000);
+  for (int idx = tid; idx < P; idx += kPrepThreads) s_sorted[idx] = idx < M ? r[idx] : __int_as_float(0x7f800000);
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int idx = tid; idx < P; idx += kCoeffThreads) {
+      for (int idx = tid; idx < P; idx += kPrepThreads) {
         const int ixj = idx ^ j;
         if (ixj > idx) {
           const float a = s_sorted[idx], c = s_sorted[ixj];
@@ -56,32 +72,31 @@ rescue_coeff_kernel(const float* __restrict__ radius, int M, int P /* pow2 >= M 
     const double a = static_cast<double>(s_sorted[lo]), c = static_cast<double>(s_sorted[hi]);
     const float q = static_cast<float>(a + (x - lo) * (c - a));
     s_q[tid] = q;
-    rq[hd * 2 + tid] = q;
+    if (blockIdx.y == 0) rq[hd * 2 + tid] = q;
   }
   __syncthreads();
   const float r_low = s_q[0], r_high = s_q[1];
   const bool live = r_high > r_low;
   const float inv = live ? 1.0f / (r_high - r_low) : 0.f;
-  auto coeff = [&](int idx) -> float {   // r_b beta_b scale of block idx (0 for padding rows); also writes beta
-    if (idx >= M) return 0.f;
-    const float rb = r[idx];
-    float bt = live ? fminf(fmaxf((rb - r_low) * inv, 0.f), 1.f) : 0.f;
-    if (beta_mode == 1) bt = 0.f;
-    if (beta_mode == 2) bt = 1.f;
-    beta[static_cast<int64_t>(hd) * M + idx] = bt;
-    return rb * bt * scale_log2;
-  };
-  // Mpad is a multiple of 128 and the loops below step by the CTA size, so every warp stays whole
-  for (int idx = tid; idx < Mpad; idx += kCoeffThreads) {
-    const uint32_t z = __ballot_sync(0xffffffffu, coeff(idx) == 0.f);
-    if (lane == 0) s_zero[idx >> 5] = static_cast<unsigned short>(__popc(z));
-  }
-  __syncthreads();
-  for (int idx = tid; idx < Mpad; idx += kCoeffThreads) {
-    const float g = coeff(idx);
+  const int row0 = static_cast<int>(blockIdx.y) * tiles_per_slice * 128, row1 = min(Mpad, row0 + tiles_per_slice * 128);
+  // groups of 1024 rows (8 tiles); Mpad and row0 are multiples of 128, so every warp stays whole
+  for (int g0 = row0; g0 < row1; g0 += kPrepThreads) {
+    const int idx = g0 + tid;
+    const bool mine = idx < row1;
+    float g = 0.f;               // r_b beta_b scale of block idx (0 for padding rows)
+    if (mine && idx < M) {
+      const float rb = r[idx];
+      float bt = live ? fminf(fmaxf((rb - r_low) * inv, 0.f), 1.f) : 0.f;
+      if (beta_mode == 1) bt = 0.f;
+      if (beta_mode == 2) bt = 1.f;
+      beta[static_cast<int64_t>(hd) * M + idx] = bt;
+      g = rb * bt * scale_log2;
+    }
     const bool zero = g == 0.f;
     const uint32_t z = __ballot_sync(0xffffffffu, zero);
-    const int tile = idx >> 7, w_in_tile = (idx >> 5) & 3;
+    if (lane == 0) s_zero[warp] = static_cast<unsigned short>(__popc(z));
+    __syncthreads();
+    const int tile = tid >> 7, w_in_tile = warp & 3;
     int zeros_tile = 0, zeros_before = 0;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
@@ -90,54 +105,47 @@ rescue_coeff_kernel(const float* __restrict__ radius, int M, int P /* pow2 >= M 
       if (w < w_in_tile) zeros_before += c;
     }
     zeros_before += __popc(z & ((1u << lane) - 1u));
-    const int before = idx & 127;                       // rows of the tile in front of this one
+    const int before = tid & 127;                       // rows of the tile in front of this one
     int pos = zero ? zeros_before : zeros_tile + (before - zeros_before);
     // odd tiles are laid out the other way round, so that the warp that gets the rows without a rescue term (half the
     // exponentials) in one tile gets the expensive rows in the next: over a query block's tiles the warps even out
-    if (tile & 1) pos = 127 - pos;
-    const int64_t dst = static_cast<int64_t>(hd) * Mpad + tile * 128 + pos;
-    gs[dst] = g;
-    perm[dst] = idx;
+    if (((idx >> 7) & 1) != 0) pos = 127 - pos;
+    const int64_t dst0 = static_cast<int64_t>(hd) * Mpad + g0;
+    if (mine) {
+      gs[dst0 + tile * 128 + pos] = g;
+      perm[dst0 + tile * 128 + pos] = idx;
+    }
+    s_dst[tid] = tile * 128 + pos;
+    __syncthreads();
+    // the group's centroids, a warp per row and four columns per lane
+    for (int rr = warp; rr < min(kPrepThreads, row1 - g0); rr += kPrepThreads / 32) {
+      const int b = g0 + rr;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (b < M) v = *reinterpret_cast<const float4*>(centroid + (static_cast<int64_t>(hd) * M + b) * kHeadDim + lane * 4);
+      v.x *= scale_log2; v.y *= scale_log2; v.z *= scale_log2; v.w *= scale_log2;
+      const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y);
+      const __nv_bfloat16 h2 = __float2bfloat16_rn(v.z), h3 = __float2bfloat16_rn(v.w);
+      const float l0 = v.x - __bfloat162float(h0), l1 = v.y - __bfloat162float(h1);
+      const float l2 = v.z - __bfloat162float(h2), l3 = v.w - __bfloat162float(h3);
+      uint2 hi, lo;
+      hi.x = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+      hi.y = static_cast<uint32_t>(__bfloat16_as_ushort(h2)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h3)) << 16);
+      lo.x = pack_bf16(l0, l1);
+      lo.y = pack_bf16(l2, l3);
+      const int64_t dst = dst0 + s_dst[rr];
+      *reinterpret_cast<uint2*>(chi + dst * kHeadDim + lane * 4) = hi;
+      *reinterpret_cast<uint2*>(clo + dst * kHeadDim + lane * 4) = lo;
+      float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      if (lane == 0) cnorm[dst] = sqrtf(n2);
+    }
+    __syncthreads();            // s_zero and s_dst may be rewritten
   }
 }
 
 // ---------------------------------------------------------------------------------------------
-// 2. fp32 centroid -> bf16 hi + bf16 lo, rows padded to Mpad with zeros
-// ---------------------------------------------------------------------------------------------
-__global__ void split_centroid_kernel(const float* __restrict__ centroid, const int* __restrict__ perm, int M, int Mpad,
-                                      int64_t n_rows_padded, float scale_log2, __nv_bfloat16* __restrict__ chi,
-                                      __nv_bfloat16* __restrict__ clo, float* __restrict__ cnorm) {
-  // One thread per 4 elements, one warp per row of the bf16 copies.  Row `row` holds block perm[row] of its
-  // (batch, KV head), multiplied by log2(e)/sqrt(d) so that the tensor-core product is the scaled logit in log2 units;
-  // also writes the row's L2 norm (of the scaled centroid).
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t row = t / (kHeadDim / 4);
-  const int c4 = static_cast<int>(t % (kHeadDim / 4));
-  if (row >= n_rows_padded) return;   // whole warps: the grid covers rows in units of 32 threads
-  const int64_t hd = row / Mpad;
-  const int b = perm[row];
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (b < M) v = *reinterpret_cast<const float4*>(centroid + (hd * M + b) * kHeadDim + c4 * 4);
-  v.x *= scale_log2; v.y *= scale_log2; v.z *= scale_log2; v.w *= scale_log2;
-  const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y);
-  const __nv_bfloat16 h2 = __float2bfloat16_rn(v.z), h3 = __float2bfloat16_rn(v.w);
-  const float l0 = v.x - __bfloat162float(h0), l1 = v.y - __bfloat162float(h1);
-  const float l2 = v.z - __bfloat162float(h2), l3 = v.w - __bfloat162float(h3);
-  uint2 hi, lo;
-  hi.x = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-  hi.y = static_cast<uint32_t>(__bfloat16_as_ushort(h2)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h3)) << 16);
-  lo.x = pack_bf16(l0, l1);
-  lo.y = pack_bf16(l2, l3);
-  *reinterpret_cast<uint2*>(chi + row * kHeadDim + c4 * 4) = hi;
-  *reinterpret_cast<uint2*>(clo + row * kHeadDim + c4 * 4) = lo;
-  float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-  if (c4 == 0) cnorm[row] = sqrtf(n2);
-}
-
-// ---------------------------------------------------------------------------------------------
-// 3. scoring + thresholds + union + pack on the 5th-generation tensor cores, one CTA per
+// 2. scoring + thresholds + union + pack on the 5th-generation tensor cores, one CTA per
 //    (batch, query head, query block), two CTAs per SM.
 //   D[128 centroids x B tokens] (fp32, tensor memory) = C_hi . Q_i^T + C_lo . Q_i^T, 16 tcgen05.mma per tile.
 //   One TMEM lane = one centroid, so the aggregation over the block's tokens is a per-thread loop over
@@ -147,7 +155,7 @@ __global__ void split_centroid_kernel(const float* __restrict__ centroid, const 
 // ---------------------------------------------------------------------------------------------
 struct SelectParams {
   const __nv_bfloat16* Q; int64_t qsb, qst, qsh;
-  // per padded centroid row, in the tile-partitioned order of rescue_coeff_kernel: bf16 hi / lo halves of the scaled
+  // per padded centroid row, in the tile-partitioned order of select_prep_kernel: bf16 hi / lo halves of the scaled
   // centroid, gs = r beta scale, norm of the scaled centroid, and the block index the row holds
   const __nv_bfloat16* chi; const __nv_bfloat16* clo; const float* gs; const float* cnorm; const int* perm;
   int M, Mpad, W, L, Hq, G, N;
@@ -155,8 +163,26 @@ struct SelectParams {
   float scale_log2, t_base, t_rescue;  // thresholds as log2(alpha)
   int n_sink, n_local, n_recent;
   uint32_t* mask; uint32_t* dbg_base; uint32_t* dbg_rescue;
-  unsigned int* counts;
+  unsigned int* counts;   // kept pairs per head: the memory of density, converted in place by the last CTA
+  unsigned int* done;     // CTAs that have finished
+  double pairs;           // causal pairs of this call
 };
+
+// The last CTA of a persistent grid to finish turns the counts into densities.  Called by one warp of the CTA, behind a
+// barrier after its last count.  (A CTA of the one-head kernel lives for one row: there the fence and the atomic at its end
+// cost 14 us in 143, more than the launch of density_kernel.)
+__device__ __forceinline__ void finish_density(const SelectParams& p, int lane) {
+  unsigned int before = 0;
+  if (lane == 0) {
+    __threadfence();
+    before = atomicAdd(p.done, 1u);
+    __threadfence();
+  }
+  if (__shfl_sync(0xffffffffu, before, 0) != gridDim.x - 1u) return;
+#pragma unroll 1
+  for (int k = lane; k < p.L * p.Hq; k += 32)
+    reinterpret_cast<float*>(p.counts)[k] = static_cast<float>(static_cast<double>(__ldcg(p.counts + k)) / p.pairs);
+}
 
 constexpr int kTcThreads = 192;
 
@@ -199,6 +225,8 @@ select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  pdl_wait();
+  pdl_trigger();
   const uint32_t tmem_base = s_tmem;
 
   if (warp == 4) {
@@ -319,8 +347,15 @@ select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   if (lane == 0 && cnt) atomicAdd(p.counts + l * p.Hq + h, cnt);
 }
 
+__global__ void density_kernel(unsigned int* __restrict__ counts, int n, double pairs) {
+  pdl_wait();
+  pdl_trigger();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < n) reinterpret_cast<float*>(counts)[t] = static_cast<float>(static_cast<double>(counts[t]) / pairs);
+}
+
 // ---------------------------------------------------------------------------------------------
-// 3b. The same scoring as a persistent kernel, one CTA per SM, that serves TWO query heads of a KV group per work
+// 2b. The same scoring as a persistent kernel, one CTA per SM, that serves TWO query heads of a KV group per work
 //     item (l, KV head, query block, head pair).  The two heads score against the same centroids, so every centroid
 //     tile is brought into shared memory once for both (half the L2 -> shared-memory traffic per score) and the
 //     tensor core runs the two heads' products back to back (four accumulators in tensor memory: 2 heads x 2 buffers).
@@ -331,7 +366,8 @@ select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 //     Warp 16: TMA producer, which also fetches the NEXT item's two Q tiles while the current item is being scored;
 //     warp 17: MMA issuer.  Each epilogue group keeps its running row maxima in registers and does its own threshold /
 //     pack pass, during which the MMA warp is already filling the accumulators of the next item.
-//     Work items are dealt round-robin, longest rows first.
+//     Work items are dealt round-robin, longest rows first.  With an odd group size the last head of a group is taken by
+//     itself, two consecutive query blocks at a time: they score against the same centroid tiles too.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPairThreads = 576;
 constexpr int kPairProducer = 16, kPairMma = 17;
@@ -339,7 +375,11 @@ constexpr int kPairProducer = 16, kPairMma = 17;
 // HALVES (blocks of 256): the two "heads" of an item are the two halves of 128 tokens of ONE head's query block; the
 // sum over the block's tokens (Eq. block_aggregation) is then the sum of the two groups' sums, handed from the second
 // group to the first like the token halves inside a group; the first group alone keeps the scores and writes the mask.
-template <int B, bool HALVES>
+// ODD: the group size is odd (a kernel of its own: as a run-time flag it cost the other group sizes 3 %).
+// FINISH: the last CTA turns the counts into densities (few items: the launch of density_kernel counts, 2 us of 16 at 1,003
+// tokens); without it the kernel is 3 % faster, whatever the reason (1.56 against 1.61 ms on the 128K layer of 32 heads;
+// same registers, no spills), so long calls launch density_kernel instead.
+template <int B, bool HALVES, bool ODD, bool FINISH>
 __global__ void __launch_bounds__(kPairThreads, 1)
 select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmChi,
                    const __grid_constant__ CUtensorMap tmClo, const SelectParams p, int n_items, int l_floats,
@@ -369,7 +409,9 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   // instead of moving every MMA operand there: 1.57 against 1.65 ms on the 128K layer of 32 heads, 6.66 against 7.33 ms on
   // the 64-head layer at blocks of 64, 0.70 against 0.77 ms at 64K.
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  const int Hkv = p.Hq / p.G, GP = HALVES ? p.G : p.G / 2;   // items per (batch, KV head, query block)
+  const int Hkv = p.Hq / p.G;
+  // items per (batch, KV head): of one query block, or of two of them when the group size is odd
+  const int GP = HALVES || ODD ? p.G : p.G / 2;
   const int per_i = p.L * Hkv * GP;
   constexpr int QB = HALVES ? 2 * B : B;                     // tokens of a query block
 
@@ -394,15 +436,41 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  pdl_wait();
+  pdl_trigger();
   const uint32_t tmem_base = s_tmem;
 
-  // item w -> (query block of the chunk, batch, KV head, head pair); longest rows first
-  auto decode = [&](int w, int& il, int& l, int& hk, int& h0) {
-    il = p.Mq - 1 - w / per_i;
+  // item w -> query blocks of the chunk and heads of its two halves, batch, KV head; longest rows first.  il[0] < 0: no
+  // such item; il[1] < 0: only the first half exists (both only in the last row pair of an odd number of query blocks)
+  struct Item { int il0, il1, l, hk, h0, h1; };
+  auto decode = [&](int w) -> Item {
+    Item it;
+    const int row = w / per_i;
     int rem = w % per_i;
     const int pr = rem % GP; rem /= GP;
-    hk = rem % Hkv; l = rem / Hkv;
-    h0 = hk * p.G + (HALVES ? pr : 2 * pr);
+    it.hk = rem % Hkv; it.l = rem / Hkv;
+    const int head0 = it.hk * p.G;
+    if (!ODD) {
+      it.il0 = it.il1 = p.Mq - 1 - row;
+      it.h0 = head0 + (HALVES ? pr : 2 * pr);
+      it.h1 = HALVES ? it.h0 : it.h0 + 1;
+    } else {
+      const int top = p.Mq - 1 - 2 * row, np = p.G >> 1;
+      if (pr == p.G - 1) {                       // the last head, two query blocks
+        it.il0 = top; it.il1 = top - 1;
+        it.h0 = it.h1 = head0 + pr;
+      } else {                                   // two heads, the pairs of the upper query block first
+        it.il0 = it.il1 = top - (pr >= np ? 1 : 0);
+        it.h0 = head0 + 2 * (pr >= np ? pr - np : pr);
+        it.h1 = it.h0 + 1;
+      }
+    }
+    return it;
+  };
+  // the next item of this CTA from w on
+  auto valid = [&](int w) -> int {
+    while (ODD && w < n_items && decode(w).il0 < 0) w += gridDim.x;
+    return w;
   };
   // tensor-memory columns of the accumulator of group hw, buffer buf: the two groups' accumulators of a buffer side by
   // side (one product writes both; HALVES reads them as one row of 2 B tokens)
@@ -415,26 +483,27 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       uint32_t nq = 0, nc = 0;     // Q loads (items) and centroid tiles issued so far
       bool ok = true;
       auto load_q = [&](int w) {
-        int il, l, hk, h0;
-        decode(w, il, l, hk, h0);
+        const Item it = decode(w);
+        const int l = it.l;
         const uint32_t slot = nq & 1;
         if (nq >= 2 && !mbar_wait(smem_u32(&bar_qempty[slot]), ((nq >> 1) - 1) & 1, status, kWaitStageFree)) { ok = false; return; }
         const uint32_t dst = smem_u32(sQ) + slot * 2 * kQTile, bar = smem_u32(&bar_qfull[slot]);
         mbar_arrive_expect_tx(bar, 2 * kQTile);
         for (int hw = 0; hw < 2; ++hw) {
-          const int hq = HALVES ? h0 : h0 + hw, tok0 = HALVES ? il * QB + hw * B : il * B;
+          const int hq = hw == 0 ? it.h0 : it.h1, il = !ODD || hw == 0 || it.il1 < 0 ? it.il0 : it.il1;
+          const int tok0 = HALVES ? il * QB + hw * B : il * B;
           tma_load_4d(dst + hw * kPanelQ, &tmQ, bar, 0, hq, tok0, l);
           tma_load_4d(dst + hw * kPanelQ + kQTile, &tmQ, bar, 64, hq, tok0, l);
         }
         ++nq;
       };
-      int w = blockIdx.x;
+      int w = valid(blockIdx.x);
       if (w < n_items) load_q(w);
-      for (; ok && w < n_items; w += gridDim.x) {
-        int il, l, hk, h0;
-        decode(w, il, l, hk, h0);
-        const int n_tiles = (p.q0 + il) / 128 + 1;
-        const int crow0 = static_cast<int>((static_cast<int64_t>(l) * Hkv + hk) * p.Mpad);
+      for (int w_next; ok && w < n_items; w = w_next) {
+        w_next = valid(w + gridDim.x);
+        const Item it = decode(w);
+        const int n_tiles = (p.q0 + it.il0) / 128 + 1;
+        const int crow0 = static_cast<int>((static_cast<int64_t>(it.l) * Hkv + it.hk) * p.Mpad);
         const uint32_t dst = smem_u32(sC);
         for (int bt = 0; ok && bt < n_tiles; ++bt, ++nc) {
           // The four 64-column panels of a centroid tile (hi 0, hi 1, lo 0, lo 1) are separate pipeline slots: a panel
@@ -447,7 +516,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           }
           if (!ok) break;
           // the next item's Q tiles go out right behind this item's first centroid tile
-          if (bt == 0 && w + static_cast<int>(gridDim.x) < n_items) load_q(w + gridDim.x);
+          if (bt == 0 && w_next < n_items) load_q(w_next);
         }
       }
     }
@@ -456,9 +525,8 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint64_t dchi = smem_desc_sw128(smem_u32(sC), 16, 1024);
     uint32_t nt = 0, k = 0;      // centroid tiles and items processed so far
     bool ok = true;
-    for (int w = blockIdx.x; ok && w < n_items; w += gridDim.x, ++k) {
-      const int il = p.Mq - 1 - w / per_i;
-      const int n_tiles = (p.q0 + il) / 128 + 1;
+    for (int w = valid(blockIdx.x); ok && w < n_items; w = valid(w + gridDim.x), ++k) {
+      const int n_tiles = (p.q0 + decode(w).il0) / 128 + 1;
       const uint32_t slot = k & 1;
       ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_qfull[slot]), (k >> 1) & 1, status, kWaitTmaFull));
       const uint64_t dq = smem_desc_sw128(smem_u32(sQ) + slot * 2 * kQTile, 16, 1024);
@@ -500,11 +568,13 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     float* sLr = sLb + l_floats;
     uint32_t nt = 0, k = 0;
     bool ok = true;
-    for (int w = blockIdx.x; ok && w < n_items; w += gridDim.x, ++k) {
-      int il, l, hk, h0;
-      decode(w, il, l, hk, h0);
-      const int i = p.q0 + il, h = HALVES ? h0 : h0 + hw;
-      const int n_tiles = i / 128 + 1;
+    for (int w = valid(blockIdx.x); ok && w < n_items; w = valid(w + gridDim.x), ++k) {
+      const Item it = decode(w);
+      const int l = it.l, hk = it.hk, h = hw == 0 ? it.h0 : it.h1;
+      const bool real = !ODD || hw == 0 || it.il1 >= 0;         // a half that does not exist repeats the first one and writes nothing
+      const int il = !ODD || hw == 0 || !real ? it.il0 : it.il1;
+      const int i = p.q0 + il;
+      const int n_tiles = (p.q0 + it.il0) / 128 + 1;    // of the item: the second half's query block may need one tile less
       const int crow0 = static_cast<int>((static_cast<int64_t>(l) * Hkv + hk) * p.Mpad);
       const uint32_t slot = k & 1;
       const unsigned char* q = sQ + slot * 2 * kQTile + hw * kPanelQ;
@@ -619,7 +689,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int64_t mrow = ((static_cast<int64_t>(l) * p.Hq + h) * p.Mq + il) * p.W;
       const bool all_forced = i >= p.M - p.n_recent;
       unsigned int cnt = 0;
-      for (int wd = wg; ok && !(HALVES && hw == 1) && wd < p.W; wd += 8) {
+      for (int wd = wg; ok && real && !(HALVES && hw == 1) && wd < p.W; wd += 8) {
         const int b = wd * 32 + lane;
         const bool valid = b <= i;
         bool kb = false, kr = false, kf = false;
@@ -648,15 +718,13 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   if (warp == kPairMma) tmem_dealloc(tmem_base, 4 * B);
+  if (FINISH && warp == kPairProducer) finish_density(p, lane);
 }
 
-__global__ void density_kernel(const unsigned int* __restrict__ counts, int n, int q0, int Mq, float* __restrict__ density) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) {
-    // causal pairs of query blocks q0 .. q0 + Mq - 1: sum of (i + 1)
-    const double pairs = static_cast<double>(Mq) * static_cast<double>(q0) + 0.5 * static_cast<double>(Mq) * static_cast<double>(Mq + 1);
-    density[t] = static_cast<float>(static_cast<double>(counts[t]) / pairs);
-  }
+static rbs_status launch_density(const SelectParams& p, cudaStream_t s) {
+  const int nh = p.L * p.Hq;
+  RBS_CUDA_OK(launch_pdl(density_kernel, (nh + 127) / 128, 1, 128, 0, s, p.counts, nh, p.pairs));
+  return RBS_OK;
 }
 
 template <int B>
@@ -676,16 +744,14 @@ static rbs_status launch_select_tc(const SelectParams& p, const rbs_tensor& Q, c
   if ((st = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem)) != RBS_OK) return st;
   const long long n_cta = static_cast<long long>(p.L) * p.Hq * p.Mq;
   if (n_cta > 0x7fffffffLL) return RBS_ERR_UNSUPPORTED;
-  kern<<<static_cast<unsigned>(n_cta), kTcThreads, smem, s>>>(tmQ, tmChi, tmClo, p, status);
-  RBS_CUDA_OK(cudaGetLastError());
-  return RBS_OK;
+  RBS_CUDA_OK(launch_pdl(kern, static_cast<unsigned>(n_cta), 1, kTcThreads, smem, s, tmQ, tmChi, tmClo, p, status));
+  return launch_density(p, s);
 }
 
 // Shared memory of select_pair_kernel for M blocks; 0 when this shape has to stay on the one-head kernel
-// (blocks of 256: two Q tiles of 64 KB each do not fit twice; an odd group size; very long rows).
+// (very long rows).
 template <int B>
 static size_t pair_kernel_smem(const SelectParams& p, int* l_floats) {
-  if (B <= 128 && p.G % 2 != 0) return 0;
   constexpr int BT = B > 128 ? 128 : B;     // tokens per Q tile (blocks of 256: two tiles of 128 of one head)
   *l_floats = (p.M + 127) / 128 * 128;
   const size_t bytes = static_cast<size_t>(4) * 128 * 128 + 4 * 2 * static_cast<size_t>(BT) * 128 + 2 * BT * sizeof(float) +
@@ -693,7 +759,7 @@ static size_t pair_kernel_smem(const SelectParams& p, int* l_floats) {
   return bytes <= 227 * 1024 - 8 * 1024 ? bytes : 0;   // up to 7 KB of static shared memory beside it
 }
 
-template <int B>
+template <int B, bool ODD, bool FINISH>
 static rbs_status launch_select_pair(const SelectParams& p, const rbs_tensor& Q, size_t smem, int l_floats, cudaStream_t s) {
   CUtensorMap tmQ, tmChi, tmClo;
   constexpr bool kHalves = B > 128;
@@ -705,13 +771,16 @@ static rbs_status launch_select_pair(const SelectParams& p, const rbs_tensor& Q,
   if ((st = make_tmap_2d(&tmClo, p.clo, rows, kHeadDim, 64, 128)) != RBS_OK) return st;
   unsigned int* status = device_status_ptr();
   if (status == nullptr) return RBS_ERR_CUDA;
-  auto kern = select_pair_kernel<BT, kHalves>;
+  auto kern = select_pair_kernel<BT, kHalves, ODD, FINISH>;
   if ((st = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem)) != RBS_OK) return st;
-  const long long n_items = static_cast<long long>(p.L) * (kHalves ? p.Hq : p.Hq / 2) * p.Mq;
+  // two heads of a query block per item; with an odd group size Hq items per two query blocks
+  const long long n_items = kHalves ? static_cast<long long>(p.L) * p.Hq * p.Mq
+                            : !ODD ? static_cast<long long>(p.L) * (p.Hq / 2) * p.Mq
+                                           : static_cast<long long>(p.L) * p.Hq * ((p.Mq + 1) / 2);
   if (n_items > 0x7fffffffLL) return RBS_ERR_UNSUPPORTED;
   const int grid = static_cast<int>(n_items < sm_count() ? n_items : sm_count());
-  kern<<<grid, kPairThreads, smem, s>>>(tmQ, tmChi, tmClo, p, static_cast<int>(n_items), l_floats, status);
-  RBS_CUDA_OK(cudaGetLastError());
+  RBS_CUDA_OK(launch_pdl(kern, grid, 1, kPairThreads, smem, s, tmQ, tmChi, tmClo, p, static_cast<int>(n_items), l_floats, status));
+  if (!FINISH) return launch_density(p, s);
   return RBS_OK;
 }
 
@@ -719,7 +788,14 @@ template <int B>
 static rbs_status launch_select(const SelectParams& p, const rbs_tensor& Q, cudaStream_t s) {
   int l_floats = 0;
   const size_t smem = pair_kernel_smem<B>(p, &l_floats);
-  if (smem != 0) return launch_select_pair<B>(p, Q, smem, l_floats, s);
+  if (smem != 0) {
+    // 2,048 scored tiles of a pair of heads: 14 per SM, about 60 us
+    const bool few = B <= 128 && static_cast<long long>(p.L) * p.Hq / 2 * p.Mq * ((p.M + 127) / 128) <= 2048;
+    constexpr bool kOdd = B <= 128, kFew = B <= 128;
+    if (kOdd && p.G % 2 != 0)
+      return few ? launch_select_pair<B, kOdd, kFew>(p, Q, smem, l_floats, s) : launch_select_pair<B, kOdd, false>(p, Q, smem, l_floats, s);
+    return few ? launch_select_pair<B, false, kFew>(p, Q, smem, l_floats, s) : launch_select_pair<B, false, false>(p, Q, smem, l_floats, s);
+  }
   return launch_select_tc<B>(p, Q, s);
 }
 
@@ -753,21 +829,23 @@ static rbs_status select_impl(const rbs_shape* shape, int q_start_block, int n_q
   float* gs = reinterpret_cast<float*>(wsp + ws.off_g);
   int* perm = reinterpret_cast<int*>(wsp + ws.off_perm);
   float* cnorm = reinterpret_cast<float*>(wsp + ws.off_cn);
-  unsigned int* counts = reinterpret_cast<unsigned int*>(wsp + ws.off_counts);
   const float scale_log2 = kLog2e / sqrtf(static_cast<float>(x.d));
 
   int P = 1;
   while (P < x.M) P <<= 1;
   if (P < 2) P = 2;
-  const size_t coeff_smem = static_cast<size_t>(P) * sizeof(float);
-  RBS_CUDA_OK(cudaMemsetAsync(counts, 0, static_cast<size_t>(x.L) * x.Hq * sizeof(unsigned int), s));
-  rescue_coeff_kernel<<<x.L * x.Hkv, kCoeffThreads, coeff_smem, s>>>(stats.radius, x.M, P, scale_log2, stats.beta,
-                                                                     stats.rq, gs, perm, ws.Mpad, beta_mode);
-  RBS_CUDA_OK(cudaGetLastError());
-  const int64_t rows = static_cast<int64_t>(x.L) * x.Hkv * ws.Mpad;
-  const int64_t n_thr = rows * (kHeadDim / 4);
-  split_centroid_kernel<<<static_cast<unsigned>((n_thr + 255) / 256), 256, 0, s>>>(stats.centroid, perm, x.M, ws.Mpad, rows, scale_log2, chi, clo, cnorm);
-  RBS_CUDA_OK(cudaGetLastError());
+  const size_t prep_smem = static_cast<size_t>(P) * sizeof(float);
+  // as many slices as bring the heads to about one CTA per SM
+  const int heads = x.L * x.Hkv, tiles = ws.Mpad / 128;
+  int slices = sm_count() / heads;
+  slices = slices < 1 ? 1 : (slices > tiles ? tiles : slices);
+  const int tiles_per_slice = (tiles + slices - 1) / slices;
+  slices = (tiles + tiles_per_slice - 1) / tiles_per_slice;
+  unsigned int* counts = reinterpret_cast<unsigned int*>(density);   // counted in place, see finish_density
+  unsigned int* done = reinterpret_cast<unsigned int*>(wsp + ws.off_counts);
+  RBS_CUDA_OK(launch_pdl(select_prep_kernel, heads, slices, kPrepThreads, prep_smem, s, stats.radius, stats.centroid, x.M, P,
+                         scale_log2, stats.beta, stats.rq, gs, perm, chi, clo, cnorm, ws.Mpad, tiles_per_slice, beta_mode,
+                         counts, x.L * x.Hq, done));
 
   SelectParams p;
   p.Q = static_cast<const __nv_bfloat16*>(Q.ptr); p.qsb = Q.stride_batch; p.qst = Q.stride_token; p.qsh = Q.stride_head;
@@ -776,13 +854,12 @@ static rbs_status select_impl(const rbs_shape* shape, int q_start_block, int n_q
   p.q0 = q_start_block; p.Nq = n_q_tokens; p.Mq = (n_q_tokens + x.B - 1) / x.B;
   p.scale_log2 = scale_log2; p.t_base = log2f(alpha_base); p.t_rescue = log2f(alpha_rescue);
   p.n_sink = n_sink; p.n_local = n_local; p.n_recent = n_recent;
-  p.mask = mask; p.dbg_base = dbg_base_mask; p.dbg_rescue = dbg_rescue_mask; p.counts = counts;
+  p.mask = mask; p.dbg_base = dbg_base_mask; p.dbg_rescue = dbg_rescue_mask; p.counts = counts; p.done = done;
+  // causal pairs of query blocks q0 .. q0 + Mq - 1: sum of (i + 1)
+  p.pairs = static_cast<double>(p.Mq) * static_cast<double>(p.q0) + 0.5 * static_cast<double>(p.Mq) * static_cast<double>(p.Mq + 1);
   if (x.B == 256) st = launch_select<256>(p, Q, s);
   else st = (x.B == 128) ? launch_select<128>(p, Q, s) : launch_select<64>(p, Q, s);
   if (st != RBS_OK) return st;
-  const int nh = x.L * x.Hq;
-  density_kernel<<<(nh + 127) / 128, 128, 0, s>>>(counts, nh, p.q0, p.Mq, density);
-  RBS_CUDA_OK(cudaGetLastError());
   return RBS_OK;
 }
 

@@ -50,6 +50,9 @@ block_stats_warp_kernel(const __grid_constant__ CUtensorMap tmK, int n_tiles, in
   }
   if (WPB == 2) __syncthreads(); else __syncwarp();
 
+  pdl_wait();
+  pdl_trigger();
+
   const int stride = gridDim.x * NG;
   int t = group * gridDim.x + blockIdx.x;
   // K is read exactly once by this pass: its lines are marked evict-first in L2 so that they do not push out what the
@@ -199,9 +202,8 @@ static rbs_status launch_stats_warp(const rbs_tensor& K, const Dims& x, const rb
   const long long n_tiles = static_cast<long long>(x.L) * x.Hkv * x.M;
   long long want = (n_tiles + NW / WPB - 1) / (NW / WPB);
   const int grid = static_cast<int>(want < sm_count() ? want : sm_count());
-  kern<<<grid, NW * 32, smem, s>>>(tm, static_cast<int>(n_tiles), x.M, x.Hkv, x.N, stats.centroid, stats.radius, box_lo,
-                                   box_hi, status);
-  RBS_CUDA_OK(cudaGetLastError());
+  RBS_CUDA_OK(launch_pdl(kern, grid, 1, NW * 32, smem, s, tm, static_cast<int>(n_tiles), x.M, x.Hkv, x.N, stats.centroid,
+                         stats.radius, box_lo, box_hi, status));
   return RBS_OK;
 }
 
