@@ -360,13 +360,17 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int per_band_kv = SCHED ? p.items_per_group : p.band_rows * p.G;
       const int per_band = p.L * Hkv * per_band_kv;
       const int n_rows = KB == 128 ? p.Mq * p.R : (p.Mq + 1) / 2;    // 128-row tiles of the call
-      int w = static_cast<int>(blockIdx.x);       // slot A's first tile; every other one is asked for
-      if (x != 0) { ask(); w = answer(); }
+      int w = x == 0 ? static_cast<int>(blockIdx.x) : -2;     // -2: to be asked for
       // a launch in which a wait has given up is lost: CTAs that start after that do nothing (looked at after the first
       // tile's mask has been requested, so that the two latencies pass together)
       uint32_t lost = *reinterpret_cast<volatile unsigned int*>(status);
 #pragma unroll 1
-      while (ok && w >= 0) {
+      while (ok) {
+        if (w == -2) {
+          if (!pending) ask();
+          w = answer();
+        }
+        if (w < 0) break;
         // Tile order: the query tiles are cut into bands of band_rows consecutive tiles, the last (longest) band first;
         // inside a band one (batch, KV head) at a time, inside it longest rows first, the G query heads of the group
         // together.  All tiles in flight then read the K/V of one KV head (64 MiB at 128K tokens), which stays in L2;
@@ -381,11 +385,8 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (SCHED) { item = __ldg(p.items + w); rem = item.x; }
         const int l = kvid / Hkv, hk = kvid % Hkv;
         const int Tl = n_rows - 1 - (band * p.band_rows + rem / p.G);
-        if ((SCHED && item.x < 0) || Tl < 0 || Tl * 128 >= p.Nq) {    // no such tile
-          ask();
-          w = answer();
-          continue;
-        }
+        w = -2;
+        if ((SCHED && item.x < 0) || Tl < 0 || Tl * 128 >= p.Nq) continue;    // no such tile
         const int h = hk * p.G + rem % p.G;
         // Q is on its way to L2 while the mask is read
         tma_prefetch_4d(&tmQ, 0, h, Tl * 128, l);
@@ -417,7 +418,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             load_k(r0, r1, begin ? info | ((pub & 1) ? kStepTileParity : 0u) : info, hk, l);
             // the next tile is asked for with the last K: the answer is there when this tile's last V is out (asked for
             // earlier, the tiles of a small grid would pile up at the first CTAs to ask)
-            if (info & kStepLast) ask();
+            if (KB == 128 && (info & kStepLast)) ask();
           }
           if (begin) {
             // A tile is announced, and its Q requested, while the one before it is under way: Q is free since that one's
@@ -429,7 +430,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (SCHED) s_part[x][pub & 1] = item.w;
             mbar_arrive(smem_u32(&bar_tile[x][pub & 1]));
             ++pub;
-            if (empty) { ask(); break; }
+            if (empty) break;
             // Q is read exactly once per launch: evict-first, so that it does not push the K/V in flight out of L2
             mbar_arrive_expect_tx(smem_u32(&bar_q[x]), kDuoTile);
             tma_load_4d_hint(q_dst, &tmQ, smem_u32(&bar_q[x]), 0, h, Tl * 128, l, pol_q);
@@ -444,9 +445,8 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           if (!ok || (!begin && (vinfo & kStepLast))) break;
           v0 = r0; v1 = r1; vinfo = info;
         }
-        w = ok ? answer() : -1;
       }
-      if (pending) (void)answer();     // (after a failure: the response must not arrive behind the CTA's end)
+      if (pending) (void)duo_wait(clc_bar, asked & 1, status, kWaitTmaFull);   // (after a failure: nothing may arrive behind the CTA's end)
       // no tile left: the issuer learns it from a step, the softmax warps from a tile
       if (ok) {
         s_step[x][nk & 3] = kStepExit;
@@ -612,112 +612,143 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           __syncwarp();
           warp_arrive(smem_u32(&bar_sfree));   // S may take the next Q K^T
           bool any = false;                    // the pair of warps has met in this step
+          // Blocks of 64: both units are first exponentiated against the maximum in use, with one check for the two; only if
+          // it fails (and in a row's first step) are they taken one after the other, each with a check of its own, as the
+          // units of blocks of 128 always are.  (Two checks per step cost 600 cycles of a step's 3,300 when a slot runs alone.)
+          bool together = KB == 64 && !first;
+          float sums[NU];
+#pragma unroll 1
+          for (;;) {
+            asm volatile("" ::: "memory");
 #pragma unroll
-          for (int u = 0; u < NU; ++u) {
-            // P of the step before has been consumed (its P V runs behind this step's Q K^T)
-            auto wait_p = [&]() {
-              ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady));
-              tc_fence_after_sync();
-            };
-            const uint32_t tp = tmem_p + u * 32;
-            if (KB == 128 || ((blk >> (4 * u + rh)) & 1u)) {     // the row's query block attends the unit's keys
-              if (KB == 128 ? (blk & 1u) : ((blk >> (4 * u + 2 + rh)) & 1u)) {   // diagonal: keys after the query are hidden
-#pragma unroll
-                for (int c = 0; c < UW; ++c)
-                  if (c > last_key) s[u * UW + c] = 0xff800000u;   // -inf
-              }
-              // 2^(s scale - m) to tensor memory as bf16 pairs; returns the sum
-              auto exps = [&]() -> float {
-                const uint64_t negm2 = f2_pack(-m_used, -m_used);
-                uint64_t sum_a = 0ull, sum_b = 0ull;   // (0.f, 0.f)
-#pragma unroll
-                for (int c0 = 0; c0 < UW; c0 += 16) {
-                  uint32_t pk[8];
-#pragma unroll
-                  for (int q = 0; q < 16; q += 4) {
-                    const int c = u * UW + c0 + q;
-                    const uint64_t x01 = f2_fma(f2_pack(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), scale2, negm2);
-                    const uint64_t x23 = f2_fma(f2_pack(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), scale2, negm2);
-                    float x0, x1, x2, x3;
-                    f2_unpack(x01, x0, x1);
-                    f2_unpack(x23, x2, x3);
-                    const float p0 = fast_exp2(x0), p1 = fast_exp2(x1), p2 = fast_exp2(x2), p3 = fast_exp2(x3);
-                    sum_a = f2_add(sum_a, f2_pack(p0, p1));
-                    sum_b = f2_add(sum_b, f2_pack(p2, p3));
-                    pk[q >> 1] = pack_bf16(p0, p1);
-                    pk[(q >> 1) + 1] = pack_bf16(p2, p3);
-                  }
-                  if (c0 == 0) wait_p();
-                  tmem_st8(tp + (c0 >> 1), pk);
-                }
-                float a0, a1, a2, a3;
-                f2_unpack(sum_a, a0, a1);
-                f2_unpack(sum_b, a2, a3);
-                return (a0 + a1) + (a2 + a3);
+            for (int u = 0; u < NU; ++u) {
+              // P of the step before has been consumed (its P V runs behind this step's Q K^T)
+              auto wait_p = [&]() {
+                ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady));
+                tc_fence_after_sync();
               };
-              // Lazy running maximum: the exponentials are first taken against the maximum in use.  Only when a sum shows
-              // that this has gone stale (sum >= kSumLimit, or not finite) is the exact maximum of the row's logits in
-              // the unit taken, O and l rescaled and the unit redone.  A row's first unit has no maximum yet and takes
-              // the exact one straight away.  The maximum is a shift that cancels in O / l: any value that keeps P
-              // finite is right.
-              float hs = 0.f;
-              bool stale = first, redo = true;
-              any = true;
-#pragma unroll 1
-              for (;;) {
-                if (!stale) {
-                  hs = exps();
-                  if (!redo) break;
-                  stale = __any_sync(0xffffffffu, !(hs < kSumLimit));
+              const uint32_t tp = tmem_p + u * 32;
+              sums[u] = 0.f;
+              if (KB == 128 || ((blk >> (4 * u + rh)) & 1u)) {     // the row's query block attends the unit's keys
+                if (KB == 128 ? (blk & 1u) : ((blk >> (4 * u + 2 + rh)) & 1u)) {   // diagonal: keys after the query are hidden
+#pragma unroll
+                  for (int c = 0; c < UW; ++c)
+                    if (c > last_key) s[u * UW + c] = 0xff800000u;   // -inf
                 }
-                if (group_all<64>(ok && !stale, pair_bar)) break;
-                ok = group_all<64>(ok, pair_bar);
-                if (!ok) break;
-                float mxa[4];
+                // 2^(s scale - m) to tensor memory as bf16 pairs; returns the sum
+                auto exps = [&]() -> float {
+                  const uint64_t negm2 = f2_pack(-m_used, -m_used);
+                  uint64_t sum_a = 0ull, sum_b = 0ull;   // (0.f, 0.f)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) mxa[v] = -INFINITY;
+                  for (int c0 = 0; c0 < UW; c0 += 16) {
+                    uint32_t pk[8];
 #pragma unroll
-                for (int c = u * UW; c < u * UW + UW; c += 8) {
-#pragma unroll
-                  for (int v = 0; v < 4; ++v) mxa[v] = max3(mxa[v], __uint_as_float(s[c + 2 * v]), __uint_as_float(s[c + 2 * v + 1]));
-                }
-                const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])) * p.scale_log2;
-                *xch_mine = mx;
-                (void)group_all<64>(true, pair_bar);
-                const float m_new = fmaxf(m_used, fmaxf(mx, *xch_other));
-                const float corr = fast_exp2(m_used - m_new);     // 0 while m_used = -inf
-                l_sum *= corr;
-                m_used = m_new;
-                if (!first) {   // O holds the P V of everything before this unit: rescale this warp's half of its columns
-                  ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady));
-                  tc_fence_after_sync();
-#pragma unroll 1
-                  for (int c0 = 0; c0 < 64; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld16(tmem_o + c0, r);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) * corr);
-                    tmem_st16(tmem_o + c0, r);
+                    for (int q = 0; q < 16; q += 4) {
+                      const int c = u * UW + c0 + q;
+                      const uint64_t x01 = f2_fma(f2_pack(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), scale2, negm2);
+                      const uint64_t x23 = f2_fma(f2_pack(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), scale2, negm2);
+                      float x0, x1, x2, x3;
+                      f2_unpack(x01, x0, x1);
+                      f2_unpack(x23, x2, x3);
+                      const float p0 = fast_exp2(x0), p1 = fast_exp2(x1), p2 = fast_exp2(x2), p3 = fast_exp2(x3);
+                      sum_a = f2_add(sum_a, f2_pack(p0, p1));
+                      sum_b = f2_add(sum_b, f2_pack(p2, p3));
+                      pk[q >> 1] = pack_bf16(p0, p1);
+                      pk[(q >> 1) + 1] = pack_bf16(p2, p3);
+                    }
+                    if (c0 == 0) wait_p();
+                    tmem_st8(tp + (c0 >> 1), pk);
                   }
+                  float a0, a1, a2, a3;
+                  f2_unpack(sum_a, a0, a1);
+                  f2_unpack(sum_b, a2, a3);
+                  return (a0 + a1) + (a2 + a3);
+                };
+                // Lazy running maximum: the exponentials are first taken against the maximum in use.  Only when a sum shows
+                // that this has gone stale (sum >= kSumLimit, or not finite) is the exact maximum of the row's logits in
+                // the unit taken, O and l rescaled and the unit redone.  A row's first unit has no maximum yet and takes
+                // the exact one straight away.  The maximum is a shift that cancels in O / l: any value that keeps P
+                // finite is right.
+                bool stale = first, redo = true;
+                any = true;
+#pragma unroll 1
+                for (;;) {
+                  if (!stale) {
+                    sums[u] = exps();
+                    if (!redo || together) break;
+                    stale = __any_sync(0xffffffffu, !(sums[u] < kSumLimit));
+                  }
+                  if (group_all<64>(ok && !stale, pair_bar)) break;
+                  ok = group_all<64>(ok, pair_bar);
+                  if (!ok) break;
+                  float mxa[4];
+#pragma unroll
+                  for (int v = 0; v < 4; ++v) mxa[v] = -INFINITY;
+#pragma unroll
+                  for (int c = u * UW; c < u * UW + UW; c += 8) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) mxa[v] = max3(mxa[v], __uint_as_float(s[c + 2 * v]), __uint_as_float(s[c + 2 * v + 1]));
+                  }
+                  const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])) * p.scale_log2;
+                  *xch_mine = mx;
+                  (void)group_all<64>(true, pair_bar);
+                  const float m_new = fmaxf(m_used, fmaxf(mx, *xch_other));
+                  const float corr = fast_exp2(m_used - m_new);     // 0 while m_used = -inf
+                  l_sum *= corr;
+                  m_used = m_new;
+                  if (!first) {   // O holds the P V of everything before this unit: rescale this warp's half of its columns
+                    ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady));
+                    tc_fence_after_sync();
+#pragma unroll 1
+                    for (int c0 = 0; c0 < 64; c0 += 16) {
+                      uint32_t r[16];
+                      tmem_ld16(tmem_o + c0, r);
+                      tmem_wait_ld();
+#pragma unroll
+                      for (int q = 0; q < 16; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) * corr);
+                      tmem_st16(tmem_o + c0, r);
+                    }
+                  }
+                  stale = false;
+                  redo = false;
                 }
-                stale = false;
-                redo = false;
+                if (!together) {
+                  first = false;
+                  l_sum += sums[u];
+                }
+              } else {
+                uint32_t zero[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) zero[q] = 0u;   // P = 0 for the rows whose block did not select these keys
+                wait_p();
+#pragma unroll
+                for (int c0 = 0; c0 < UW / 2; c0 += 8) tmem_st8(tp + c0, zero);
               }
-              first = false;
-              l_sum += hs;
-            } else {
-              uint32_t zero[8];
-#pragma unroll
-              for (int q = 0; q < 8; ++q) zero[q] = 0u;   // P = 0 for the rows whose block did not select these keys
-              wait_p();
-#pragma unroll
-              for (int c0 = 0; c0 < UW / 2; c0 += 8) tmem_st8(tp + c0, zero);
+              if (!together) {
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                warp_arrive(smem_u32(&bar_in[x][u]));
+              }
             }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            __syncwarp();
-            warp_arrive(smem_u32(&bar_in[x][u]));
+            if (!together) break;
+            bool good = true;
+#pragma unroll
+            for (int u = 0; u < NU; ++u) good = good && sums[u] < kSumLimit;
+            good = __all_sync(0xffffffffu, good);
+            if (!any || group_all<64>(ok && good, pair_bar)) {
+#pragma unroll
+              for (int u = 0; u < NU; ++u) l_sum += sums[u];
+              tmem_wait_st();
+              tc_fence_before_sync();
+              __syncwarp();
+#pragma unroll
+              for (int u = 0; u < NU; ++u) warp_arrive(smem_u32(&bar_in[x][u]));
+              break;
+            }
+            ok = group_all<64>(ok, pair_bar);
+            if (!ok) break;
+            together = false;
           }
           if (KB == 64 && !any) ok = group_all<64>(ok, pair_bar);
           if (!ok) break;
