@@ -30,14 +30,14 @@ import torch
 # DRAM bytes (read + write) of one rbs_sparse_prefill launch from an ncu capture of that workload at the default
 # thresholds: (bytes, where the capture is summarised).  A workload without a capture reports null and says so.
 NCU_TRAFFIC_BYTES = {
-    "q30b_128k": (4623220000 + 1038194000, "profiles/prefill_tc_kernel_q30b_128k.md"),
-    "q30b_32k": (455600000 + 232200000, "profiles/prefill_tc_kernel_q30b_32k.md"),
+    "q30b_128k": (4477247232 + 1024324096, "profiles/prefill_duo_kernel_q30b.md"),
+    "q30b_32k": (443410176 + 216024064, "profiles/prefill_duo_kernel_q30b.md"),
 }
 NOMINAL_BF16_TFLOPS = 2250.0     # dense bf16 per B200, for context next to the measured peak
 TARGET_TENSOR_FRAC = 0.60        # select + sparse attention on the selected FLOPs, of the measured bf16 peak
 TARGET_HBM_FRAC = 0.70           # statistics pass, of the measured copy bandwidth
-# kernels per step of the path: block_stats; select_prep, select_pair; prefill_duo
-LAUNCHES_PER_STEP = 4
+# kernels per step of the path: block_stats; select_prep, select_pair, density; prefill_duo
+LAUNCHES_PER_STEP = 5
 # the bounded oracle sample both arms time (the same in `cpu_baseline` and in `--impl reference`)
 ORACLE_SAMPLE = dict(n_heads=4, n_att_rows=48)
 

@@ -321,8 +321,8 @@ def rbs_select_box(Q: torch.Tensor, box_lo: torch.Tensor, box_hi: torch.Tensor, 
 
 def rbs_sparse_prefill_grouped(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, mask: torch.Tensor, block: int, *,
                                out: torch.Tensor | None = None, return_lse: bool = False, softmax_scale: float = 0.0):
-    """rbs_sparse_prefill for masks that are identical inside every KV group (after rbs_mask_group_union): two heads
-    of a group share one stream of K/V tiles."""
+    """rbs_sparse_prefill for masks that are identical inside every KV group (after rbs_mask_group_union): the mask row
+    of the first head of each pair is read, and the heads of a group run next to each other."""
     lib = load_library()
     L, N, Hq, d = Q.shape
     shape = RbsShape(L, N, Hq, K.shape[2], d, block)

@@ -51,19 +51,6 @@ __device__ __forceinline__ int next_block(const uint32_t* __restrict__ row, int 
   return -1;
 }
 
-// Tensor-core path, blocks of R x 128 tokens: the kernel works on 128-row query tiles T and 128-key sub-blocks kb.
-// Sub-block kb belongs to mask block kb / R; tile T (of query block T / R) attends sub-blocks kb <= T of the selected
-// blocks, kb == T being the diagonal one.  Returns the next sub-block after `cur` (-1 to start), or -1.
-__device__ __forceinline__ int next_kb(const uint32_t* __restrict__ row, int cur, int i, int R, int T) {
-  int kb = cur + 1;
-  if (kb > T) return -1;
-  const int b = kb / R;
-  const int nb = next_block(row, b - 1, i);   // first selected block >= b
-  if (nb < 0) return -1;
-  if (nb != b) kb = nb * R;
-  return kb <= T ? kb : -1;
-}
-
 // A half-row of P whose sum reaches this value makes the row adopt the half's exact maximum (the lazy running maximum
 // of the tensor-core kernels).
 constexpr float kSumLimit = 16384.0f;

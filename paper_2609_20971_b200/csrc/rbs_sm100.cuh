@@ -173,17 +173,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
@@ -379,54 +368,6 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
-}
-
-__device__ __forceinline__ uint64_t f2_add_rm(uint64_t a, uint64_t b) {   // round toward -inf
-  uint64_t d;
-  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-// 2^x for two values on the FMA pipe instead of the special-function unit (which is the scarce unit in
-// the softmax): x = n + f with n = floor(x), 2^f by a degree-3 minimax polynomial on [0, 1) (relative
-// error 7.5e-5), then n is added into the exponent field.  Inputs are clamped to x >= -126; x <= 127.
-__device__ __forceinline__ void exp2_poly_x2(uint64_t x2, float& r0, float& r1) {
-  constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: its float spacing is 1
-  float x0, x1;
-  f2_unpack(x2, x0, x1);
-  const uint64_t xc = f2_pack(fmaxf(x0, -126.0f), fmaxf(x1, -126.0f));
-  const uint64_t t = f2_add_rm(xc, f2_pack(kMagic, kMagic));                  // low mantissa bits = floor(x)
-  const uint64_t fl = f2_add(t, f2_pack(-kMagic, -kMagic));                   // floor(x), exact
-  const uint64_t f = f2_fma(fl, f2_pack(-1.0f, -1.0f), xc);                   // x - floor(x) in [0, 1)
-  uint64_t pl = f2_fma(f, f2_pack(0.0780242234f, 0.0780242234f), f2_pack(0.2260672301f, 0.2260672301f));
-  pl = f2_fma(pl, f, f2_pack(0.6958336830f, 0.6958336830f));
-  pl = f2_fma(pl, f, f2_pack(0.9999251962f, 0.9999251962f));
-  float p0, p1, t0, t1;
-  f2_unpack(pl, p0, p1);
-  f2_unpack(t, t0, t1);
-  r0 = __int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23));
-  r1 = __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23));
-}
-
-// Same idea without the clamp, for callers that know -126 <= x <= 127, and with a degree-4 polynomial
-// (relative error 2.6e-6).  Everything runs on the FMA pipe: the exponent is added with an integer multiply-add.
-__device__ __forceinline__ void exp2_poly4_x2(uint64_t x2, float& r0, float& r1) {
-  constexpr float kMagic = 12582912.0f;
-  const uint64_t t = f2_add_rm(x2, f2_pack(kMagic, kMagic));
-  const uint64_t fl = f2_add(t, f2_pack(-kMagic, -kMagic));
-  const uint64_t f = f2_fma(fl, f2_pack(-1.0f, -1.0f), x2);
-  uint64_t pl = f2_fma(f, f2_pack(0.0135341408f, 0.0135341408f), f2_pack(0.0520114899f, 0.0520114899f));
-  pl = f2_fma(pl, f, f2_pack(0.2414427549f, 0.2414427549f));
-  pl = f2_fma(pl, f, f2_pack(0.6930038333f, 0.6930038333f));
-  pl = f2_fma(pl, f, f2_pack(1.0000026226f, 1.0000026226f));
-  float p0, p1, t0, t1;
-  f2_unpack(pl, p0, p1);
-  f2_unpack(t, t0, t1);
-  int b0, b1;
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(b0) : "r"(__float_as_int(t0)), "r"(__float_as_int(p0)));
-  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(b1) : "r"(__float_as_int(t1)), "r"(__float_as_int(p1)));
-  r0 = __int_as_float(b0);
-  r1 = __int_as_float(b1);
 }
 
 }  // namespace rbs
