@@ -46,25 +46,25 @@ enum : uint32_t { kStepLast = 1u << 8, kStepOneHalf = 1u << 9, kStepTileParity =
 enum : int { kTileExit = 1, kTileEmpty = 2 };
 struct DuoTileInfo { int Tl, h, l, flags; };
 
-// mbar_wait (rbs_sm100.cuh) for this kernel: the waiting thread is suspended for up to kWaitHintNs per probe instead of
-// probing all the time (twenty warps share the issue slots with the exponentials), and the loop is a handful of
-// instructions without divergence handling.  Bounded: about a second in all, then `code` goes to the status word.
-constexpr uint32_t kWaitHintNs = 20000, kWaitProbes = 50000;
+// mbar_wait (rbs_sm100.cuh) for this kernel in a handful of instructions without divergence handling (the hot loops of the
+// roles share the instruction caches, and it waits in some twenty places).  A probe that fails has suspended the thread for
+// 4 us (measured; a longer hint changes nothing).  Bounded: about a second in all, then `code` goes to the status word.
+constexpr uint32_t kWaitProbes = 250000;
 __device__ __forceinline__ bool duo_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .u32 c;\n\t"
       "mov.u32 c, 0;\n"
       "WAIT:\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "@p bra.uni DONE;\n\t"
       "add.u32 c, c, 1;\n\t"
-      "setp.lt.u32 p, c, %4;\n\t"
+      "setp.lt.u32 p, c, %3;\n\t"
       "@p bra.uni WAIT;\n\t"
       "setp.ne.u32 p, 0, 0;\n"
       "DONE:\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "n"(kWaitHintNs), "n"(kWaitProbes) : "memory");
+      : "=r"(ok) : "r"(bar), "r"(parity), "n"(kWaitProbes) : "memory");
   if (ok == 0u) atomicCAS(status, 0u, code);
   return ok != 0u;
 }
