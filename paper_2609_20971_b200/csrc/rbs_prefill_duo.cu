@@ -86,6 +86,9 @@ __device__ __forceinline__ void warp_tell(uint32_t word, uint32_t value, uint32_
       ::"r"(word), "r"(value), "r"(bar) : "memory");
 }
 
+// What warp 18 does without a turn before it gives up (64 ns and two probes each: about a second too).
+constexpr uint32_t kIdleTurns = 1u << 22;
+
 // An mbarrier probe that does not wait.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -275,7 +278,6 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (uint32_t it = 0; it < kSpinLimit; ++it) {
           if (atomicCAS(&s_lock, 0u, 1u) == 0u) { __threadfence_block(); return true; }
           if (it > 64) __nanosleep(64);
-          if ((it & 255u) == 255u && *reinterpret_cast<volatile unsigned int*>(status) != 0u) break;
         }
         atomicCAS(status, 0u, static_cast<unsigned int>(kWaitStageFree));
         return false;
@@ -361,9 +363,6 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int per_band = p.L * Hkv * per_band_kv;
       const int n_rows = KB == 128 ? p.Mq * p.R : (p.Mq + 1) / 2;    // 128-row tiles of the call
       int w = x == 0 ? static_cast<int>(blockIdx.x) : -2;     // -2: to be asked for
-      // a launch in which a wait has given up is lost: CTAs that start after that do nothing (looked at after the first
-      // tile's mask has been requested, so that the two latencies pass together)
-      uint32_t lost = *reinterpret_cast<volatile unsigned int*>(status);
 #pragma unroll 1
       while (ok) {
         if (w == -2) {
@@ -406,7 +405,6 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           walk.start(-1, 0);
         }
         const bool empty = !walk.any();
-        if (lost != 0u) break;
         int r0 = 0, r1 = 0, v0 = 0, v1 = 0;
         uint32_t info = 0, vinfo = 0;
         bool first_v = true;
@@ -446,7 +444,13 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           v0 = r0; v1 = r1; vinfo = info;
         }
       }
-      if (pending) (void)duo_wait(clc_bar, asked & 1, status, kWaitTmaFull);   // (after a failure: nothing may arrive behind the CTA's end)
+      // A launch in which a wait has given up is lost: the CTAs that have not started are cancelled and their tiles dropped,
+      // so that it ends within seconds.  (The status word cannot say so: it outlives the launch.)
+      if (!ok) {
+        if (!pending) ask();
+        while (answer() >= 0) ask();
+      }
+      if (pending) (void)answer();   // nothing may arrive behind the CTA's end
       // no tile left: the issuer learns it from a step, the softmax warps from a tile
       if (ok) {
         s_step[x][nk & 3] = kStepExit;
@@ -518,7 +522,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const bool b = ok && turn(std::integral_constant<int, 1>());
       if (a || b) { idle = 0; continue; }
       if (++idle > 2048) __nanosleep(64);
-      if ((idle & 255u) == 255u && (*reinterpret_cast<volatile unsigned int*>(status) != 0u || idle >= kSpinLimit)) {
+      if (idle >= kIdleTurns) {
         atomicCAS(status, 0u, static_cast<unsigned int>(kWaitTmaFull));
         ok = false;
       }

@@ -43,6 +43,11 @@ for kw in cases:
     out[cfg.name] = dict(centroid=st.centroid.cpu(), radius=st.radius.cpu(), mask=mask.cpu(), O=O.cpu(), Od=Od.cpu())
 # a check that fails by construction: recorded, its access skipped, nothing traps, and the library works afterwards
 flag = rbs_selftest_debug_check()
+for kw in cases:         # ... also while the failed check is still recorded
+    cfg = SynthConfig(**kw)
+    Q, K, V = (t.cuda() for t in make_inputs(cfg))
+    O = rbs_sparse_prefill(Q, K, V, out[cfg.name]["mask"].cuda(), cfg.B)
+    assert torch.equal(O.cpu(), out[cfg.name]["O"])
 code = rbs_device_status(clear=True)
 assert flag is not None and int(flag.item()) == 1 and code == 0x1ff, (flag, hex(code))
 cfg = SynthConfig(**cases[0])

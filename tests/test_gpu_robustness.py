@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import rbs_oracle as orc
-from paper_2609_20971_b200 import rbs_block_stats, rbs_device_status
+from paper_2609_20971_b200 import rbs_block_stats, rbs_device_status, rbs_select, rbs_sparse_prefill
 from paper_2609_20971_b200.binding import rbs_selftest_wait_timeout
 from paper_2609_20971_b200.synth import SynthConfig, make_inputs, to_f64
 
@@ -33,3 +33,29 @@ def test_wait_that_runs_out_reports_and_leaves_the_context_usable():
         assert np.allclose(st.centroid[0, hk].cpu().numpy(), c, rtol=2e-5, atol=2e-6)
         assert np.allclose(st.radius[0, hk].cpu().numpy(), r, rtol=2e-5)
     assert rbs_device_status(clear=True) == 0
+
+
+@pytest.mark.parametrize("B", [64, 128, 256])
+def test_a_recorded_time_out_leaves_later_calls_alone(B):
+    """The status word belongs to the launch that wrote it: calls issued while it still holds a code give the bits they
+    give without one, and leave the code for whoever reads it."""
+    from paper_2609_20971_b200.binding import prefill_workspace_bytes
+    cfg = SynthConfig("sticky", N=B * 21 + 37, Hq=4, Hkv=2, B=B, sigma=(0.1, 1.0), seed=91)
+    Q, K, V = (t.cuda() for t in make_inputs(cfg))
+    ws = torch.empty(max(256, prefill_workspace_bytes(1, cfg.N, cfg.Hq, cfg.Hkv, B)), dtype=torch.uint8, device="cuda")
+
+    def path():
+        st = rbs_block_stats(K, B)
+        mask, dens = rbs_select(Q, st, B)
+        outs = []
+        for m, w in ((mask, None), (mask, ws), (None, None)):
+            out = torch.full_like(Q, 7.0)
+            outs += [*rbs_sparse_prefill(Q, K, V, m, B, out=out, return_lse=True, workspace=w)]
+        torch.cuda.synchronize()
+        return [st.centroid, st.radius, st.beta, mask, dens, *outs]
+    assert rbs_device_status(clear=True) == 0
+    want = path()
+    rbs_selftest_wait_timeout(4096)
+    got = path()
+    assert rbs_device_status(clear=True) == WAIT_SELFTEST_CODE
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
