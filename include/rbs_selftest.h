@@ -30,6 +30,15 @@ RBS_API int rbs_selftest_device_table(void);
 RBS_API rbs_status rbs_selftest_wait_timeout(unsigned int spin_limit, unsigned int* gave_up, void* stream);
 
 /*
+ * Launches one warp on `stream` that runs the attention kernel's two forms of the bounded wait, with 1,024 probes each
+ * (about 4 ms), on a barrier whose phase is complete and on one that nothing arrives on.  answers (device, four
+ * uint32): the lanes that saw the first barrier (all of them) and the second (none), then the same two answers of one
+ * lane waiting alone (1, 0).  Afterwards rbs_device_status() reports RBS_ERR_TIMEOUT until cleared, and the CUDA context
+ * is fully usable.  Returns RBS_ERR_INVALID_ARG for a null pointer.
+ */
+RBS_API rbs_status rbs_selftest_warp_wait(unsigned int* answers, void* stream);
+
+/*
  * Debug build only (the library compiled with -DRBS_DEBUG; rbs_version() says "debug checks"): launches one thread
  * on `stream` that runs one of the kernels' index checks with an index equal to its bound.  The check fails, records
  * 0x100 + 0xff in the device status word and the guarded access is skipped: afterwards *skipped (device, one

@@ -94,6 +94,8 @@ def load_library() -> ctypes.CDLL:
     lib.rbs_selftest_device_table.argtypes = []
     lib.rbs_selftest_wait_timeout.restype = i
     lib.rbs_selftest_wait_timeout.argtypes = [ctypes.c_uint, vp, vp]
+    lib.rbs_selftest_warp_wait.restype = i
+    lib.rbs_selftest_warp_wait.argtypes = [vp, vp]
     lib.rbs_selftest_debug_check.restype = i
     lib.rbs_selftest_debug_check.argtypes = [vp, vp]
     lib.rbs_status_string.restype = ctypes.c_char_p
@@ -170,6 +172,14 @@ def rbs_selftest_wait_timeout(spin_limit: int = 4096) -> torch.Tensor:
     flag = torch.zeros(1, dtype=torch.int32, device="cuda")
     _check(load_library().rbs_selftest_wait_timeout(spin_limit, _ptr(flag), _stream()), "rbs_selftest_wait_timeout")
     return flag
+
+
+def rbs_selftest_warp_wait() -> torch.Tensor:
+    """Launches the self-test of the attention kernel's waits (one warp; a barrier that is complete and one nothing
+    arrives on) and returns the four words it writes.  The status word then holds the code."""
+    answers = torch.zeros(4, dtype=torch.int32, device="cuda")
+    _check(load_library().rbs_selftest_warp_wait(_ptr(answers), _stream()), "rbs_selftest_warp_wait")
+    return answers
 
 
 def rbs_selftest_debug_check() -> torch.Tensor | None:

@@ -46,27 +46,13 @@ enum : uint32_t { kStepLast = 1u << 8, kStepOneHalf = 1u << 9, kStepTileParity =
 enum : int { kTileExit = 1, kTileEmpty = 2 };
 struct DuoTileInfo { int Tl, h, l, flags; };
 
-// mbar_wait (rbs_sm100.cuh) for this kernel in a handful of instructions without divergence handling (the hot loops of the
-// roles share the instruction caches, and it waits in some twenty places).  A probe that fails has suspended the thread for
-// 4 us (measured; a longer hint changes nothing).  Bounded: about a second in all, then `code` goes to the status word.
+// About a second: a probe that fails has suspended its warp for 4 us (measured; a longer hint changes nothing).
 constexpr uint32_t kWaitProbes = 250000;
-__device__ __forceinline__ bool duo_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .u32 c;\n\t"
-      "mov.u32 c, 0;\n"
-      "WAIT:\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "@p bra.uni DONE;\n\t"
-      "add.u32 c, c, 1;\n\t"
-      "setp.lt.u32 p, c, %3;\n\t"
-      "@p bra.uni WAIT;\n\t"
-      "setp.ne.u32 p, 0, 0;\n"
-      "DONE:\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "n"(kWaitProbes) : "memory");
-  if (ok == 0u) atomicCAS(status, 0u, code);
-  return ok != 0u;
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
+  return warp_wait_probes<kWaitProbes>(bar, parity, status, code);
+}
+__device__ __forceinline__ bool lane_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
+  return lane_wait_probes<kWaitProbes>(bar, parity, status, code);
 }
 // one arrival by a converged warp
 __device__ __forceinline__ void warp_arrive(uint32_t bar) {
@@ -298,7 +284,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       auto answer = [&]() -> int {
         if (!pending) return -1;
         pending = false;
-        if (!duo_wait(clc_bar, asked & 1, status, kWaitTmaFull)) return -1;
+        if (!lane_wait(clc_bar, asked & 1, status, kWaitTmaFull)) return -1;
         ++asked;
         if (!lock()) return -1;
         uint32_t got, cx;
@@ -328,7 +314,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           // panel 0 of this parity was freed by the step before last, whose phase was waited for with the last panel 1
-          if (c == 1) ok = duo_wait(smem_u32(&bar_s[x]), (nk - 1) & 1, status, kWaitStageFree);
+          if (c == 1) ok = lane_wait(smem_u32(&bar_s[x]), (nk - 1) & 1, status, kWaitStageFree);
           if (!ok) return;
           const uint32_t dst = kv_dst + (c == 0 ? (nk & 1) : 2) * kDuoStage;
           if (KB == 128) {
@@ -347,7 +333,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const uint32_t dst = kv_dst + 3 * kDuoStage;
 #pragma unroll
         for (int u = 0; u < (KB == 128 ? 1 : 2); ++u) {
-          ok = ok && duo_wait(smem_u32(&bar_pv[x][u]), (nv - 1) & 1, status, kWaitStageFree);
+          ok = ok && lane_wait(smem_u32(&bar_pv[x][u]), (nv - 1) & 1, status, kWaitStageFree);
           if (!ok) return;
           const uint32_t bar = smem_u32(&bar_in[x][u]);
           if (u == 1 && (info & kStepOneHalf)) {
@@ -422,7 +408,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             // A tile is announced, and its Q requested, while the one before it is under way: Q is free since that one's
             // last Q K^T (the wait for K panel 1).  The tile before that is done: its ofree has been waited for, with the
             // first V of the tile before this one, or here.
-            if (empty) ok = duo_wait(smem_u32(&bar_ofree[x]), (pub - 1) & 1, status, kWaitStageFree);
+            if (empty) ok = lane_wait(smem_u32(&bar_ofree[x]), (pub - 1) & 1, status, kWaitStageFree);
             if (!ok) break;
             s_tile[x][pub & 1] = DuoTileInfo{Tl, h, l, empty ? kTileEmpty : 0};
             if (SCHED) s_part[x][pub & 1] = item.w;
@@ -435,7 +421,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tma_load_4d_hint(q_dst + kDuoPanel, &tmQ, smem_u32(&bar_q[x]), 64, h, Tl * 128, l, pol_q);
           } else if (ok) {
             if (first_v) {     // the V buffer takes the output of the tile before
-              ok = duo_wait(smem_u32(&bar_ofree[x]), pub & 1, status, kWaitStageFree);
+              ok = lane_wait(smem_u32(&bar_ofree[x]), pub & 1, status, kWaitStageFree);
               first_v = false;
             }
             if (ok) load_v(v0, v1, vinfo, hk, l);
@@ -489,7 +475,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       }
       const uint32_t kbar = smem_u32(&bar_k[X][n[X] & 1]), kph = (n[X] >> 1) & 1;
       if (mid[X]) {
-        ok = __all_sync(0xffffffffu, duo_wait(kbar, kph, status, kWaitTmaFull));
+        ok = warp_wait(kbar, kph, status, kWaitTmaFull);
         if (!ok) return false;
       } else if (!__all_sync(0xffffffffu, mbar_test(kbar, kph))) {
         return false;
@@ -502,7 +488,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                          mbar_test(smem_u32(&bar_tdone[X]), (info & kStepTileParity) ? 0u : 1u))) return false;
         ++tiles[X];
       }
-      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_sfree), (uses - 1) & 1, status, kWaitTmemFree));
+      ok = warp_wait(smem_u32(&bar_sfree), (uses - 1) & 1, status, kWaitTmemFree);
       if (!ok) return false;
       tc_fence_after_sync();
       if (n[X] & 1) mma_ss_k64_commit_elect(tmem_s, dq + kQ, dk + kKV + kStage16, kIdescQK, 0, 0);
@@ -543,12 +529,12 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       constexpr uint64_t kV = static_cast<uint64_t>(X * kDuoStages + 3) * kStage16;
       const uint32_t info = *reinterpret_cast<volatile uint32_t*>(&s_step[X][n[X] & 3]);
       const uint32_t ph = n[X] & 1;
-      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_in[X][0]), ph, status, kWaitPReady));
+      ok = warp_wait(smem_u32(&bar_in[X][0]), ph, status, kWaitPReady);
       if (!ok) return;
       tc_fence_after_sync();
       mma_ts_k64_elect(tmem + X * 128, tmem + 384 + X * 64, dv + kV, kIdescPV, 2048 >> 4, !first[X], KB == 64 ? smem_u32(&bar_pv[X][0]) : 0u);
       if (KB == 64) {
-        ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_in[X][1]), ph, status, kWaitPReady));
+        ok = warp_wait(smem_u32(&bar_in[X][1]), ph, status, kWaitPReady);
         if (!ok) return;
         tc_fence_after_sync();
       }
@@ -559,7 +545,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     };
 #pragma unroll 1
     for (uint32_t turns = 0; ok; ++turns) {
-      ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_turn[turns & 7]), (turns >> 3) & 1, status, kWaitPReady));
+      ok = warp_wait(smem_u32(&bar_turn[turns & 7]), (turns >> 3) & 1, status, kWaitPReady);
       if (!ok) break;
       const uint32_t what = *reinterpret_cast<volatile uint32_t*>(&s_turn[turns & 7]);
       if (what == 0u) product(std::integral_constant<int, 0>());
@@ -589,7 +575,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     // together.
 #pragma unroll 1
     for (;;) {
-      bool ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_tile[x][tiles & 1]), (tiles >> 1) & 1, status, kWaitTmaFull));
+      bool ok = warp_wait(smem_u32(&bar_tile[x][tiles & 1]), (tiles >> 1) & 1, status, kWaitTmaFull);
       const DuoTileInfo ti = s_tile[x][tiles & 1];
       const int part_slot = SCHED ? s_part[x][tiles & 1] : -1;
       bool store = false;
@@ -600,7 +586,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         bool first = true;                       // the row has attended nothing yet
 #pragma unroll 1
         for (bool more = !(ti.flags & kTileEmpty); more; ++n) {
-          ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_s[x]), n & 1, status, kWaitMmaDone));
+          ok = warp_wait(smem_u32(&bar_s[x]), n & 1, status, kWaitMmaDone);
           const uint32_t blk = *reinterpret_cast<volatile uint32_t*>(&s_step[x][n & 3]);
           more = (blk & kStepLast) == 0u;
           tc_fence_after_sync();
@@ -628,7 +614,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             for (int u = 0; u < NU; ++u) {
               // P of the step before has been consumed (its P V runs behind this step's Q K^T)
               auto wait_p = [&]() {
-                ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady));
+                ok = ok && warp_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady);
                 tc_fence_after_sync();
               };
               const uint32_t tp = tmem_p + u * 32;
@@ -701,7 +687,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                   l_sum *= corr;
                   m_used = m_new;
                   if (!first) {   // O holds the P V of everything before this unit: rescale this warp's half of its columns
-                    ok = __all_sync(0xffffffffu, duo_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady));
+                    ok = warp_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady);
                     tc_fence_after_sync();
 #pragma unroll 1
                     for (int c0 = 0; c0 < 64; c0 += 16) {
@@ -769,7 +755,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (lse_dst && hf == 0) *lse_dst = -INFINITY;
           }
         } else {
-          ok = __all_sync(0xffffffffu, ok && duo_wait(smem_u32(&bar_pv[x][NU - 1]), (n - 1) & 1, status, kWaitOReady));
+          ok = ok && warp_wait(smem_u32(&bar_pv[x][NU - 1]), (n - 1) & 1, status, kWaitOReady);
           tc_fence_after_sync();
           *xch_mine = l_sum;
           ok = group_all<64>(ok, pair_bar);

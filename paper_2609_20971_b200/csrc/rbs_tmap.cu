@@ -136,6 +136,27 @@ __global__ void selftest_wait_kernel(unsigned int* status, unsigned int spin_lim
   *gave_up = ok ? 0u : 1u;
 }
 
+// One warp and the waits of the attention kernel, 1,024 probes (4 ms) each: on a barrier whose phase is complete and on one
+// that nothing arrives on.  answers: the lanes whose wait succeeded, for either barrier; the same of lane 0 waiting alone.
+__global__ void selftest_warp_wait_kernel(unsigned int* status, unsigned int* answers) {
+  __shared__ __align__(8) uint64_t there, never;
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&there), 1);
+    mbar_init(smem_u32(&never), 1);
+    mbar_fence_init();
+    mbar_arrive(smem_u32(&there));
+  }
+  __syncwarp();
+  const unsigned int a = __ballot_sync(0xffffffffu, warp_wait_probes<1024>(smem_u32(&there), 0, status, kWaitSelfTest));
+  const unsigned int b = __ballot_sync(0xffffffffu, warp_wait_probes<1024>(smem_u32(&never), 0, status, kWaitSelfTest));
+  if (threadIdx.x == 0) {
+    answers[0] = a;
+    answers[1] = b;
+    answers[2] = lane_wait_probes<1024>(smem_u32(&there), 0, status, kWaitSelfTest) ? 1u : 0u;
+    answers[3] = lane_wait_probes<1024>(smem_u32(&never), 0, status, kWaitSelfTest) ? 1u : 0u;
+  }
+}
+
 }  // namespace rbs
 
 extern "C" rbs_status rbs_device_status(void* stream, unsigned int* code_out, int clear) {
@@ -183,6 +204,15 @@ extern "C" rbs_status rbs_selftest_wait_timeout(unsigned int spin_limit, unsigne
   unsigned int* status = rbs::device_status_ptr();
   if (status == nullptr) return RBS_ERR_CUDA;
   rbs::selftest_wait_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(status, spin_limit, gave_up);
+  RBS_CUDA_OK(cudaGetLastError());
+  return RBS_OK;
+}
+
+extern "C" rbs_status rbs_selftest_warp_wait(unsigned int* answers, void* stream) {
+  if (answers == nullptr) return RBS_ERR_INVALID_ARG;
+  unsigned int* status = rbs::device_status_ptr();
+  if (status == nullptr) return RBS_ERR_CUDA;
+  rbs::selftest_warp_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(status, answers);
   RBS_CUDA_OK(cudaGetLastError());
   return RBS_OK;
 }

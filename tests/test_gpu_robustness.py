@@ -35,6 +35,15 @@ def test_wait_that_runs_out_reports_and_leaves_the_context_usable():
     assert rbs_device_status(clear=True) == 0
 
 
+def test_waits_of_a_whole_warp_give_every_lane_the_same_answer():
+    from paper_2609_20971_b200.binding import rbs_selftest_warp_wait
+    assert rbs_device_status(clear=True) == 0
+    for _ in range(5):
+        answers = [int(x) & 0xffffffff for x in rbs_selftest_warp_wait().tolist()]
+        assert answers == [0xffffffff, 0, 1, 0]
+        assert rbs_device_status(clear=True) == WAIT_SELFTEST_CODE
+
+
 @pytest.mark.parametrize("B", [64, 128, 256])
 def test_a_recorded_time_out_leaves_later_calls_alone(B):
     """The status word belongs to the launch that wrote it: calls issued while it still holds a code give the bits they
