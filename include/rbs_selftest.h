@@ -47,6 +47,17 @@ RBS_API rbs_status rbs_selftest_warp_wait(unsigned int* answers, void* stream);
  */
 RBS_API rbs_status rbs_selftest_debug_check(unsigned int* skipped, void* stream);
 
+/*
+ * Debug build only: makes one wait of the attention kernel run out in every thread block of the attention calls that
+ * follow.  Softmax warp `warp` (0 .. 15; negative: no wait any more) does its wait of the kind `which` (0: the next tile's
+ * announcement, 1: S of a step, 2: P free, 3: O before it is rescaled, 4: O of a tile) that has `before` waits of that
+ * kind in front of it on a barrier that nothing arrives on, with 64 probes.  Such a call ends within seconds with its
+ * outputs undefined and code 7 in the status word; nothing traps or faults, and once the switch is back at -1 and the
+ * word cleared, calls are as before.  Synchronous; not for use beside running attention calls.  The release build
+ * returns RBS_ERR_UNSUPPORTED.
+ */
+RBS_API rbs_status rbs_selftest_attention_wait(int warp, int which, int before);
+
 #ifdef __cplusplus
 }
 #endif

@@ -96,6 +96,8 @@ def load_library() -> ctypes.CDLL:
     lib.rbs_selftest_wait_timeout.argtypes = [ctypes.c_uint, vp, vp]
     lib.rbs_selftest_warp_wait.restype = i
     lib.rbs_selftest_warp_wait.argtypes = [vp, vp]
+    lib.rbs_selftest_attention_wait.restype = i
+    lib.rbs_selftest_attention_wait.argtypes = [i, i, i]
     lib.rbs_selftest_debug_check.restype = i
     lib.rbs_selftest_debug_check.argtypes = [vp, vp]
     lib.rbs_status_string.restype = ctypes.c_char_p
@@ -192,6 +194,16 @@ def rbs_selftest_debug_check() -> torch.Tensor | None:
         return None
     _check(rc, "rbs_selftest_debug_check")
     return flag
+
+
+def rbs_selftest_attention_wait(warp: int, which: int = 0, before: int = 0) -> bool:
+    """Debug library only: makes one wait of one softmax warp run out in the attention calls that follow (warp < 0: none
+    any more).  False in the release library, which has no such switch."""
+    rc = load_library().rbs_selftest_attention_wait(warp, which, before)
+    if rc == 2:       # RBS_ERR_UNSUPPORTED: release build
+        return False
+    _check(rc, "rbs_selftest_attention_wait")
+    return True
 
 
 def rbs_version() -> str:

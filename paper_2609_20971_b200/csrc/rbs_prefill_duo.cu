@@ -28,6 +28,7 @@
 
 #include "rbs_prefill.cuh"
 #include "rbs_score.cuh"
+#include "rbs_selftest.h"
 
 namespace rbs {
 
@@ -54,6 +55,13 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, unsigne
 __device__ __forceinline__ bool lane_wait(uint32_t bar, uint32_t parity, unsigned int* status, unsigned int code) {
   return lane_wait_probes<kWaitProbes>(bar, parity, status, code);
 }
+// The waits of the softmax warps, by what they wait for.
+enum : int { kSoftTile = 0, kSoftS = 1, kSoftP = 2, kSoftRescale = 3, kSoftO = 4 };
+#ifdef RBS_DEBUG
+// rbs_selftest_attention_wait: {softmax warp (-1: none), which of its waits, how many of those come before}: that wait is
+// done on a barrier that nothing arrives on, with 64 probes.
+__device__ int g_selftest_wait[3] = {-1, 0, 0};
+#endif
 // one arrival by a converged warp
 __device__ __forceinline__ void warp_arrive(uint32_t bar) {
   asm volatile(
@@ -216,6 +224,9 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __shared__ DuoTileInfo s_tile[2][2];           // [slot][tile parity]
   __shared__ int s_part[2][2];
   __shared__ uint32_t s_tmem, s_lock, s_no_more;
+#ifdef RBS_DEBUG
+  __shared__ __align__(8) uint64_t bar_never;
+#endif
 
   const int tid = threadIdx.x, lane = tid & 31;
   // uniform for the compiler: the roles then run on uniform registers and branches (20 % less code, 55 instead of 128 moves
@@ -235,6 +246,9 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
     for (int k = 0; k < 8; ++k) mbar_init(smem_u32(&bar_turn[k]), 1);
     mbar_init(smem_u32(&bar_sfree), 8);
+#ifdef RBS_DEBUG
+    mbar_init(smem_u32(&bar_never), 1);
+#endif
     s_lock = 0; s_no_more = 0;
     mbar_fence_init();
   }
@@ -570,12 +584,24 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     float* const xch_mine = &s_xch[x][hf][row];
     const float* const xch_other = &s_xch[x][hf ^ 1][row];
     uint32_t n = 0, tiles = 0;
-    // Every warp of the slot passes the barrier at the end of the loop once per tile, and the two warps of a pair meet at
-    // least once per step, also when a wait has given up: `ok` goes through the barriers, so that warps leave the loops
-    // together.
+#ifdef RBS_DEBUG
+    const int st_which = g_selftest_wait[0] == warp ? g_selftest_wait[1] : -1;
+    int st_before = g_selftest_wait[2];
+#endif
+    auto wait = [&](int which, uint64_t* bar, uint32_t parity, unsigned int code) -> bool {
+#ifdef RBS_DEBUG
+      if (which == st_which && st_before-- == 0) return warp_wait_probes<64>(smem_u32(&bar_never), 0, status, kWaitSelfTest);
+#endif
+      return warp_wait(smem_u32(bar), parity, status, code);
+    };
+    // Named barriers have no limit, so a wait that gives up in one warp must not part it from the others.  Every warp of the
+    // slot passes the barrier at the end of the loop once per tile.  The two warps of a pair pass the same barriers: both
+    // enter a tile or none does; a warp that has given up inside a tile keeps that to itself (`ok`) until the next
+    // barriers of the pair, and only what both have learned there, behind two barriers of a step, ends the tile
+    // (`lost`).  A warp whose wait for a step gave up does not know the step's barriers: it passes two and is out.
 #pragma unroll 1
     for (;;) {
-      bool ok = warp_wait(smem_u32(&bar_tile[x][tiles & 1]), (tiles >> 1) & 1, status, kWaitTmaFull);
+      bool ok = group_all<64>(wait(kSoftTile, &bar_tile[x][tiles & 1], (tiles >> 1) & 1, kWaitTmaFull), pair_bar);
       const DuoTileInfo ti = s_tile[x][tiles & 1];
       const int part_slot = SCHED ? s_part[x][tiles & 1] : -1;
       bool store = false;
@@ -586,7 +612,12 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         bool first = true;                       // the row has attended nothing yet
 #pragma unroll 1
         for (bool more = !(ti.flags & kTileEmpty); more; ++n) {
-          ok = warp_wait(smem_u32(&bar_s[x]), n & 1, status, kWaitMmaDone);
+          ok = ok && wait(kSoftS, &bar_s[x], n & 1, kWaitMmaDone);
+          if (!ok) {
+            (void)group_all<64>(false, pair_bar);
+            (void)group_all<64>(false, pair_bar);
+            goto lost;
+          }
           const uint32_t blk = *reinterpret_cast<volatile uint32_t*>(&s_step[x][n & 3]);
           more = (blk & kStepLast) == 0u;
           tc_fence_after_sync();
@@ -614,7 +645,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             for (int u = 0; u < NU; ++u) {
               // P of the step before has been consumed (its P V runs behind this step's Q K^T)
               auto wait_p = [&]() {
-                ok = ok && warp_wait(smem_u32(&bar_pv[x][u]), (n - 1) & 1, status, kWaitOReady);
+                ok = ok && wait(kSoftP, &bar_pv[x][u], (n - 1) & 1, kWaitOReady);
                 tc_fence_after_sync();
               };
               const uint32_t tp = tmem_p + u * 32;
@@ -669,8 +700,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     stale = __any_sync(0xffffffffu, !(sums[u] < kSumLimit));
                   }
                   if (group_all<64>(ok && !stale, pair_bar)) break;
-                  ok = group_all<64>(ok, pair_bar);
-                  if (!ok) break;
+                  if (!group_all<64>(ok, pair_bar)) goto lost;
                   float mxa[4];
 #pragma unroll
                   for (int v = 0; v < 4; ++v) mxa[v] = -INFINITY;
@@ -687,7 +717,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                   l_sum *= corr;
                   m_used = m_new;
                   if (!first) {   // O holds the P V of everything before this unit: rescale this warp's half of its columns
-                    ok = warp_wait(smem_u32(&bar_pv[x][u == 0 ? NU - 1 : 0]), (u == 0 ? n - 1 : n) & 1, status, kWaitOReady);
+                    ok = ok && wait(kSoftRescale, &bar_pv[x][u == 0 ? NU - 1 : 0], (u == 0 ? n - 1 : n) & 1, kWaitOReady);
                     tc_fence_after_sync();
 #pragma unroll 1
                     for (int c0 = 0; c0 < 64; c0 += 16) {
@@ -736,12 +766,17 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
               for (int u = 0; u < NU; ++u) warp_arrive(smem_u32(&bar_in[x][u]));
               break;
             }
-            ok = group_all<64>(ok, pair_bar);
-            if (!ok) break;
+            if (!group_all<64>(ok, pair_bar)) goto lost;
             together = false;
           }
-          if (KB == 64 && !any) ok = group_all<64>(ok, pair_bar);
-          if (!ok) break;
+          if (KB == 64 && !any && !group_all<64>(ok, pair_bar)) {
+            (void)group_all<64>(false, pair_bar);
+            goto lost;
+          }
+        }
+        if (false) {
+        lost:
+          ok = false;
         }
         // epilogue: O / l -> bf16 -> global
         const int tok = ti.Tl * 128 + row;
@@ -755,7 +790,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (lse_dst && hf == 0) *lse_dst = -INFINITY;
           }
         } else {
-          ok = ok && warp_wait(smem_u32(&bar_pv[x][NU - 1]), (n - 1) & 1, status, kWaitOReady);
+          ok = ok && wait(kSoftO, &bar_pv[x][NU - 1], (n - 1) & 1, kWaitOReady);
           tc_fence_after_sync();
           *xch_mine = l_sum;
           ok = group_all<64>(ok, pair_bar);
@@ -855,3 +890,15 @@ rbs_status launch_prefill_duo(const PrefillParams& p, const rbs_tensor& Q, const
 }
 
 }  // namespace rbs
+
+extern "C" rbs_status rbs_selftest_attention_wait(int warp, int which, int before) {
+#ifdef RBS_DEBUG
+  if (warp > 15 || which < 0 || which > rbs::kSoftO || before < 0) return RBS_ERR_INVALID_ARG;
+  const int v[3] = {warp < 0 ? -1 : warp, which, before};
+  RBS_CUDA_OK(cudaMemcpyToSymbol(rbs::g_selftest_wait, v, sizeof(v)));
+  return RBS_OK;
+#else
+  (void)warp; (void)which; (void)before;
+  return RBS_ERR_UNSUPPORTED;   // the release build has no such switch
+#endif
+}

@@ -85,3 +85,60 @@ def test_debug_library_runs_the_path_clean_and_bit_identical(tmp_path):
         assert torch.equal(st.centroid.cpu(), g["centroid"]) and torch.equal(st.radius.cpu(), g["radius"])
         assert torch.equal(mask.cpu(), g["mask"])
         assert torch.equal(O.cpu(), g["O"]) and torch.equal(Od.cpu(), g["Od"])
+
+
+WAIT_CHILD = r"""
+import sys, time, torch
+from paper_2609_20971_b200 import rbs_sparse_prefill, rbs_device_status
+from paper_2609_20971_b200.binding import prefill_workspace_bytes, rbs_selftest_attention_wait
+N, Hq, Hkv = 64 * 80 - 20, 16, 2
+g = torch.Generator(device="cuda").manual_seed(5)
+Q, K, V = (torch.randn(1, N, h, 128, generator=g, device="cuda") for h in (Hq, Hkv, Hkv))
+K += 0.05 * torch.arange(N, device="cuda").view(1, N, 1, 1) / 64     # logits that grow: maxima go stale all the time
+Q += 0.5
+Q, K, V = Q.bfloat16(), K.bfloat16(), V.bfloat16()
+ws = torch.empty(prefill_workspace_bytes(1, N, Hq, Hkv, 128), dtype=torch.uint8, device="cuda")
+def call(B, schedule):
+    M = (N + B - 1) // B
+    mask = torch.full((1, Hq, M, (M + 31) // 32), -1, dtype=torch.int32, device="cuda")
+    return rbs_sparse_prefill(Q, K, V, mask, B, out=torch.zeros_like(Q), workspace=ws if schedule else None)
+want = {k: call(*k) for k in ((64, False), (128, False), (128, True))}
+assert rbs_device_status(clear=True) == 0
+for B, schedule, warp, which, before in eval(sys.argv[1]):
+    assert rbs_selftest_attention_wait(warp, which, before)
+    t = time.time()
+    call(B, schedule)
+    torch.cuda.synchronize()
+    t = time.time() - t
+    code = rbs_device_status(clear=True)
+    assert rbs_selftest_attention_wait(-1)
+    print("case", B, schedule, warp, which, before, "%.2f s" % t, flush=True)
+    assert code == 7 and t < 20.0, code
+    for k in want:
+        assert torch.equal(call(*k), want[k])
+    assert rbs_device_status(clear=True) == 0
+print("wait child ok")
+"""
+
+# (block, schedule, warp, which of its waits, how many of them before): both slots, both key halves, a tile's first step (exact
+# maximum) and later ones, blocks of 64 with one and with two checks
+WAITS = [
+    (128, False, 0, 0, 0), (128, False, 5, 0, 2), (128, False, 0, 1, 0), (128, False, 13, 1, 4), (128, False, 4, 2, 1),
+    (128, False, 9, 3, 0), (128, False, 0, 4, 0), (128, True, 6, 1, 2),
+    (64, False, 0, 0, 1), (64, False, 5, 1, 0), (64, False, 8, 1, 3), (64, False, 2, 2, 0), (64, False, 4, 2, 5),
+    (64, False, 1, 3, 1), (64, False, 12, 4, 1),
+]
+
+
+def test_a_softmax_warp_whose_wait_runs_out_takes_the_launch_to_its_end():
+    """One warp of the attention kernel gives up a wait (it is done on a barrier that nothing arrives on) while the warp it
+    shares its rows with goes on: the launch must still end, report the code, and leave later calls as before.  Without
+    agreement between the two about which barriers come next the launch would not end."""
+    from paper_2609_20971_b200.binding import rbs_selftest_attention_wait
+    from paper_2609_20971_b200.build import build_library
+    assert rbs_selftest_attention_wait(0) is False        # the release library has no such switch
+    build_library(debug=True)
+    env = dict(os.environ, RBS_DEBUG="1", PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    r = subprocess.run([sys.executable, "-c", WAIT_CHILD, repr(WAITS)], env=env, cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and "wait child ok" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
