@@ -377,7 +377,7 @@ constexpr double kRowOrderBytes = 40.0 * 1024 * 1024;
 static int tile_bands(int n_rows, bool scheduled, double kv_bytes) {
   if (!scheduled && kv_bytes <= kRowOrderBytes) return n_rows;
   const int n_bands = n_rows / 64;
-  return n_bands < 1 ? 1 : (n_bands > 4 ? 4 : n_bands);
+  return n_bands < 1 ? 1 : (n_bands > kMaxBands ? kMaxBands : n_bands);
 }
 
 static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q, const rbs_tensor& K,

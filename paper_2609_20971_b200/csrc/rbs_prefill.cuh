@@ -32,6 +32,7 @@ struct PrefillParams {
 // merged afterwards; the cut depends only on the row itself, so a row is treated the same in every call.
 constexpr int kSplitCap = 256;
 constexpr int kSplitMaxParts = 4;      // parts per split row
+constexpr int kMaxBands = 4;           // bands of the scheduled tile order
 constexpr int kSplitRowsPerGroup = 8;  // split rows per (band, batch, KV head) group: its longest ones
 constexpr int kSplitSlotsPerGroup = kSplitRowsPerGroup * kSplitMaxParts;
 constexpr int kExtraItemsPerGroup = kSplitRowsPerGroup * (kSplitMaxParts - 1);

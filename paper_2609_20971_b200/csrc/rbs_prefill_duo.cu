@@ -152,6 +152,7 @@ struct StepWalk<128> {
     if (two && (kb & 1) && cur == kb - 1) next();             // a part that starts in the middle of a block
   }
   __device__ __forceinline__ bool any() const { return cur >= 0; }
+  __device__ __forceinline__ int last_row() const { return Tw * 128; }   // first key row of the last sub-block
   // the current step: first key row of its two halves of 64 keys, flags; then moves on
   __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
     r0 = cur * 128; r1 = r0 + 64;
@@ -188,6 +189,7 @@ struct StepWalk<64> {
   }
   __device__ __forceinline__ void start(int, int) { load(0); ua = ub = 0u; next(); }
   __device__ __forceinline__ bool any() const { return cur >= 0; }
+  __device__ __forceinline__ int last_row() const { return iB * 64; }
   __device__ __forceinline__ uint32_t take(int& r0, int& r1) {
     r0 = cur * 64;
     uint32_t f = f_cur;
@@ -393,12 +395,13 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         StepWalk<KB> walk;
         if constexpr (KB == 128) {
           const int T = p.q0 * p.R + Tl, i = T / p.R;
-          if (!RBS_DBG_OK(i >= p.q0 && i - p.q0 < p.Mq && h < p.Hq && l < p.L && T < p.M * p.R, status, kDbgPrefillTile)) break;
+          if (!RBS_DBG_OK(i >= p.q0 && i - p.q0 < p.Mq && h < p.Hq && l < p.L && T < p.M * p.R, status, kDbgPrefillTile)) continue;
           walk.row = p.mask ? p.mask + ((static_cast<int64_t>(l) * p.Hq + h - rem % p.G % p.mask_heads) * p.Mq + (i - p.q0)) * p.W : nullptr;
           walk.i = i; walk.T = T;
           walk.Tw = SCHED ? min(T, item.z - 1) : T;
           walk.start(SCHED ? item.y - 1 : -1, p.R);
         } else {
+          if (!RBS_DBG_OK(2 * Tl < p.Mq && h < p.Hq && l < p.L && p.q0 + 2 * Tl < p.M, status, kDbgPrefillTile)) continue;
           walk.iA = p.q0 + 2 * Tl; walk.iB = walk.iA + 1;
           walk.rowA = p.mask + ((static_cast<int64_t>(l) * p.Hq + h) * p.Mq + 2 * Tl) * p.W;
           walk.rowB = (2 * Tl + 1 < p.Mq) ? walk.rowA + p.W : nullptr;
@@ -412,7 +415,10 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (bool begin = true;; begin = false) {   // the K of a step in front of the V of the step before it
           if (begin ? !empty : !(vinfo & kStepLast)) {
             info = walk.take(r0, r1);
-            if (!RBS_DBG_OK(r0 < p.N, status, kDbgPrefillBlock)) { ok = false; break; }
+            // (a key block that fails the check is replaced by the first one: the step goes on and nobody waits)
+            const bool two = KB == 64 && !(info & kStepOneHalf);
+            if (!RBS_DBG_OK(r0 >= 0 && r0 <= walk.last_row() && r0 < p.N, status, kDbgPrefillBlock)) r0 = 0;
+            if (two && !RBS_DBG_OK(r1 > r0 && r1 <= walk.last_row() && r1 < p.N, status, kDbgPrefillBlock)) r1 = 0;
             load_k(r0, r1, begin ? info | ((pub & 1) ? kStepTileParity : 0u) : info, hk, l);
             // the next tile is asked for with the last K: the answer is there when this tile's last V is out (asked for
             // earlier, the tiles of a small grid would pile up at the first CTAs to ask)
@@ -798,9 +804,10 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           if (SCHED && part_slot >= 0) {
             // a part of a split row: the unnormalised O row, the maximum in use and the row sum go to the part's slot;
             // combine_parts_kernel merges the parts of the row in a fixed order
+            const bool room = RBS_DBG_OK(part_slot < kMaxBands * p.L * (p.Hq / p.G) * kSplitSlotsPerGroup, status, kDbgPrefillPart);
             float* po = p.part_o + (static_cast<int64_t>(part_slot) * 128 + row) * 128 + hf * 64;
 #pragma unroll 1
-            for (int c0 = 0; ok && c0 < 64; c0 += 32) {
+            for (int c0 = 0; ok && room && c0 < 64; c0 += 32) {
               uint32_t r[32];
               tmem_ld32(tmem_o + c0, r);
               tmem_wait_ld();
@@ -808,7 +815,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
               for (int q = 0; q < 32; q += 4)
                 *reinterpret_cast<uint4*>(po + c0 + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
             }
-            if (ok && hf == 0) {
+            if (ok && room && hf == 0) {
               float* ml = p.part_ml + static_cast<int64_t>(part_slot) * 256;
               ml[row] = m_used;
               ml[128 + row] = l_sum;

@@ -12,7 +12,7 @@ import pytest
 import torch
 
 from paper_2609_20971_b200 import rbs_block_stats, rbs_select, rbs_sparse_prefill
-from paper_2609_20971_b200.binding import rbs_selftest_debug_check, rbs_version
+from paper_2609_20971_b200.binding import prefill_workspace_bytes, rbs_selftest_debug_check, rbs_version
 from paper_2609_20971_b200.synth import SynthConfig, make_inputs
 
 pytestmark = pytest.mark.gpu
@@ -23,12 +23,13 @@ CASES = [
     dict(name="dbg_b64", N=64 * 70 + 9, Hq=2, Hkv=1, B=64, sigma=0.5, seed=91),
     dict(name="dbg_b128", L=2, N=128 * 37 + 50, Hq=4, Hkv=2, B=128, sigma=(0.1, 1.0), seed=92),
     dict(name="dbg_b256", N=256 * 7 + 200, Hq=3, Hkv=1, B=256, sigma=(0.1, 1.0), s_q=3.5, seed=93),
+    dict(name="dbg_split", N=128 * 300 + 77, Hq=2, Hkv=1, B=128, sigma=(0.1, 1.0), seed=94, n_recent=2),   # rows cut into parts
 ]
 
 CHILD = r"""
 import sys, torch
 from paper_2609_20971_b200 import rbs_block_stats, rbs_select, rbs_sparse_prefill, rbs_device_status
-from paper_2609_20971_b200.binding import rbs_version, rbs_selftest_debug_check
+from paper_2609_20971_b200.binding import prefill_workspace_bytes, rbs_version, rbs_selftest_debug_check
 from paper_2609_20971_b200.synth import SynthConfig, make_inputs
 assert "debug checks" in rbs_version(), rbs_version()
 cases = eval(sys.argv[1]); out = {}
@@ -36,11 +37,13 @@ for kw in cases:
     cfg = SynthConfig(**kw)
     Q, K, V = (t.cuda() for t in make_inputs(cfg))
     st = rbs_block_stats(K, cfg.B)
-    mask, dens = rbs_select(Q, st, cfg.B, cfg.alpha_base, cfg.alpha_rescue, 1, 1, 1)
+    mask, dens = rbs_select(Q, st, cfg.B, cfg.alpha_base, cfg.alpha_rescue, 1, 1, cfg.n_recent)
     O = rbs_sparse_prefill(Q, K, V, mask, cfg.B)
     Od = rbs_sparse_prefill(Q, K, V, None, cfg.B)
+    ws = torch.empty(max(256, prefill_workspace_bytes(cfg.L, cfg.N, cfg.Hq, cfg.Hkv, cfg.B)), dtype=torch.uint8, device="cuda")
+    Os = rbs_sparse_prefill(Q, K, V, mask, cfg.B, workspace=ws)
     assert rbs_device_status(clear=True) == 0, "a device-side check or wait failed on " + cfg.name
-    out[cfg.name] = dict(centroid=st.centroid.cpu(), radius=st.radius.cpu(), mask=mask.cpu(), O=O.cpu(), Od=Od.cpu())
+    out[cfg.name] = dict(centroid=st.centroid.cpu(), radius=st.radius.cpu(), mask=mask.cpu(), O=O.cpu(), Od=Od.cpu(), Os=Os.cpu())
 # a check that fails by construction: recorded, its access skipped, nothing traps, and the library works afterwards
 flag = rbs_selftest_debug_check()
 for kw in cases:         # ... also while the failed check is still recorded
@@ -78,13 +81,16 @@ def test_debug_library_runs_the_path_clean_and_bit_identical(tmp_path):
         cfg = SynthConfig(**kw)
         Q, K, V = (t.cuda() for t in make_inputs(cfg))
         st = rbs_block_stats(K, cfg.B)
-        mask, _ = rbs_select(Q, st, cfg.B, cfg.alpha_base, cfg.alpha_rescue, 1, 1, 1)
+        mask, _ = rbs_select(Q, st, cfg.B, cfg.alpha_base, cfg.alpha_rescue, 1, 1, cfg.n_recent)
         O = rbs_sparse_prefill(Q, K, V, mask, cfg.B)
         Od = rbs_sparse_prefill(Q, K, V, None, cfg.B)
+        ws = torch.empty(max(256, prefill_workspace_bytes(cfg.L, cfg.N, cfg.Hq, cfg.Hkv, cfg.B)), dtype=torch.uint8, device="cuda")
+        Os = rbs_sparse_prefill(Q, K, V, mask, cfg.B, workspace=ws)
         g = got[cfg.name]
         assert torch.equal(st.centroid.cpu(), g["centroid"]) and torch.equal(st.radius.cpu(), g["radius"])
         assert torch.equal(mask.cpu(), g["mask"])
         assert torch.equal(O.cpu(), g["O"]) and torch.equal(Od.cpu(), g["Od"])
+        assert torch.equal(Os.cpu(), g["Os"])
 
 
 WAIT_CHILD = r"""
