@@ -21,6 +21,13 @@ extern "C" {
 RBS_API int rbs_selftest_device_table(void);
 
 /*
+ * Host only, needs no GPU.  The number of kernels that rbs_select (n_q_tokens = seqlen) or rbs_select_chunk launches for
+ * this shape: 2 where the scoring kernel turns its counts into densities itself (short calls at blocks of 64 and 128),
+ * else 3; 0 for a shape that is refused.
+ */
+RBS_API int rbs_selftest_select_launches(const rbs_shape* shape, int n_q_tokens);
+
+/*
  * Launches one single-thread CTA on `stream` that waits, with the library's bounded mbarrier wait, on a barrier
  * that nothing ever arrives on, with `spin_limit` probes (1 .. 65536) instead of the production limit.  The wait
  * runs out, records its code in the device status word and the kernel returns normally: afterwards

@@ -92,6 +92,8 @@ def load_library() -> ctypes.CDLL:
     lib.rbs_select_box.argtypes = [ctypes.POINTER(RbsShape), RbsTensor, RbsBox, ctypes.c_double, i, i, i, vp, vp, vp, vp, sz, vp]
     lib.rbs_selftest_device_table.restype = i
     lib.rbs_selftest_device_table.argtypes = []
+    lib.rbs_selftest_select_launches.restype = i
+    lib.rbs_selftest_select_launches.argtypes = [ctypes.POINTER(RbsShape), i]
     lib.rbs_selftest_wait_timeout.restype = i
     lib.rbs_selftest_wait_timeout.argtypes = [ctypes.c_uint, vp, vp]
     lib.rbs_selftest_warp_wait.restype = i

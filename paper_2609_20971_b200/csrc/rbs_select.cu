@@ -10,6 +10,7 @@
 #include "rbs_common.cuh"
 #include "rbs_sm100.cuh"
 #include "rbs_score.cuh"
+#include "rbs_selftest.h"
 
 namespace rbs {
 
@@ -376,9 +377,7 @@ constexpr int kPairProducer = 16, kPairMma = 17;
 // sum over the block's tokens (Eq. block_aggregation) is then the sum of the two groups' sums, handed from the second
 // group to the first like the token halves inside a group; the first group alone keeps the scores and writes the mask.
 // ODD: the group size is odd (a kernel of its own: as a run-time flag it cost the other group sizes 3 %).
-// FINISH: the last CTA turns the counts into densities (few items: the launch of density_kernel counts, 2 us of 16 at 1,003
-// tokens); without it the kernel is 3 % faster, whatever the reason (1.56 against 1.61 ms on the 128K layer of 32 heads;
-// same registers, no spills), so long calls launch density_kernel instead.
+// FINISH: the last CTA turns the counts into densities instead of density_kernel (see finishes_itself).
 template <int B, bool HALVES, bool ODD, bool FINISH>
 __global__ void __launch_bounds__(kPairThreads, 1)
 select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmChi,
@@ -750,10 +749,9 @@ static rbs_status launch_select_tc(const SelectParams& p, const rbs_tensor& Q, c
 
 // Shared memory of select_pair_kernel for M blocks; 0 when this shape has to stay on the one-head kernel
 // (very long rows).
-template <int B>
-static size_t pair_kernel_smem(const SelectParams& p, int* l_floats) {
-  constexpr int BT = B > 128 ? 128 : B;     // tokens per Q tile (blocks of 256: two tiles of 128 of one head)
-  *l_floats = (p.M + 127) / 128 * 128;
+static size_t pair_kernel_smem(int B, int M, int* l_floats) {
+  const int BT = B > 128 ? 128 : B;     // tokens per Q tile (blocks of 256: two tiles of 128 of one head)
+  *l_floats = (M + 127) / 128 * 128;
   const size_t bytes = static_cast<size_t>(4) * 128 * 128 + 4 * 2 * static_cast<size_t>(BT) * 128 + 2 * BT * sizeof(float) +
                        4 * static_cast<size_t>(*l_floats) * sizeof(float);
   return bytes <= 227 * 1024 - 8 * 1024 ? bytes : 0;   // up to 7 KB of static shared memory beside it
@@ -784,13 +782,22 @@ static rbs_status launch_select_pair(const SelectParams& p, const rbs_tensor& Q,
   return RBS_OK;
 }
 
+// Whether the scoring kernel turns the counts into densities itself: up to 4,096 scored tiles (query block of one head x 128
+// key blocks), at blocks of 64 and 128.  What it saves is a launch between this kernel and attention; what it costs is a
+// slower scoring kernel.  Whole passes with it / without: 1,003 tokens of 32 heads (256 tiles) 41.8 / 44.0 us, 2,048 tokens of
+// 64 heads at blocks of 64 (2,048 tiles) 108 / 110, 16K of 32 heads (4,096) 627 / 630, 32K (16,384) 1,655 / 1,658, 114,688
+// tokens of one head at blocks of 64 (25,088) 1,363 / 1,366, the last two within the runs' difference.  rbs_select alone,
+// call after call, is slower with it: 14.8 / 14.0, 36.8 / 33.4, 82.8 / 80.7, 191 / 186, 141 / 125.
+static bool finishes_itself(int B, int L, int Hq, int Mq, int M) {
+  return B <= 128 && static_cast<long long>(L) * Hq * Mq * ((M + 127) / 128) <= 4096;
+}
+
 template <int B>
 static rbs_status launch_select(const SelectParams& p, const rbs_tensor& Q, cudaStream_t s) {
   int l_floats = 0;
-  const size_t smem = pair_kernel_smem<B>(p, &l_floats);
+  const size_t smem = pair_kernel_smem(B, p.M, &l_floats);
   if (smem != 0) {
-    // 2,048 scored tiles of a pair of heads: 14 per SM, about 60 us
-    const bool few = B <= 128 && static_cast<long long>(p.L) * p.Hq / 2 * p.Mq * ((p.M + 127) / 128) <= 2048;
+    const bool few = finishes_itself(B, p.L, p.Hq, p.Mq, p.M);
     constexpr bool kOdd = B <= 128, kFew = B <= 128;
     if (kOdd && p.G % 2 != 0)
       return few ? launch_select_pair<B, kOdd, kFew>(p, Q, smem, l_floats, s) : launch_select_pair<B, kOdd, false>(p, Q, smem, l_floats, s);
@@ -898,6 +905,15 @@ extern "C" rbs_status rbs_select_variant(const rbs_shape* shape, rbs_tensor Q, r
                          dbg_base_mask, dbg_rescue_mask, workspace, workspace_bytes, stream);
   }
   return RBS_ERR_INVALID_ARG;
+}
+
+extern "C" int rbs_selftest_select_launches(const rbs_shape* shape, int n_q_tokens) {
+  using namespace rbs;
+  if (check_shape(shape) != RBS_OK || n_q_tokens <= 0 || n_q_tokens > shape->seqlen) return 0;
+  const Dims x = make_dims(*shape);
+  int l_floats = 0;
+  const bool pair = pair_kernel_smem(x.B, x.M, &l_floats) != 0;
+  return pair && finishes_itself(x.B, x.L, x.Hq, (n_q_tokens + x.B - 1) / x.B, x.M) ? 2 : 3;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -204,3 +204,22 @@ def test_grouped_prefill_and_box_selector_argument_checks(lib):
     assert call(good, 0.05, need - 1) == WORKSPACE
     assert call(RbsShape(1, 1024, 4, 2, 128, 256), 0.05) == UNSUPPORTED
     assert lib.rbs_block_stats_box(ctypes.byref(good), t, _stats(), binding.RbsBox(0, 0x1000), None) == INVALID
+
+
+@pytest.mark.parametrize("shape, n_q, want", [
+    ((1, 4096, 1, 1, 128, 64), 4096, 2),           # 64 tiles of one head
+    ((1, 1003, 32, 4, 128, 128), 1003, 2),
+    ((1, 16384, 32, 4, 128, 128), 16384, 2),       # 4,096 tiles
+    ((1, 16385, 32, 4, 128, 128), 16385, 3),       # 32 * 129 * 2
+    ((1, 114688, 1, 1, 128, 64), 114688, 3),       # one head of any length is not a short call: 1,792 * 14 tiles
+    ((1, 114688, 1, 1, 128, 64), 4096, 2),         # a chunk of it is
+    ((3, 65536, 1, 1, 128, 128), 65536, 3),        # 3 * 512 * 4
+    ((1, 2048, 4, 2, 128, 256), 2048, 3),          # blocks of 256
+    ((1, 128 * 1664, 1, 1, 128, 128), 128, 2),     # rows of up to 1,664 blocks fit the two-head kernel (64: 5,760) ...
+    ((1, 128 * 1665, 1, 1, 128, 128), 128, 3),     # ... longer ones do not
+    ((1, 64 * 5760, 1, 1, 128, 64), 64, 2),
+    ((1, 64 * 5761, 1, 1, 128, 64), 64, 3),
+    ((1, 1024, 3, 2, 128, 128), 1024, 0),
+])
+def test_launches_of_a_selection(lib, shape, n_q, want):
+    assert lib.rbs_selftest_select_launches(ctypes.byref(RbsShape(*shape)), n_q) == want
