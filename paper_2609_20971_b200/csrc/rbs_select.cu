@@ -180,6 +180,8 @@ __device__ __forceinline__ void finish_density(const SelectParams& p, int lane) 
     __threadfence();
   }
   if (__shfl_sync(0xffffffffu, before, 0) != gridDim.x - 1u) return;
+  __syncwarp();          // (a shuffle orders no memory: the other lanes' reads come behind lane 0's fence through this)
+  __threadfence();
 #pragma unroll 1
   for (int k = lane; k < p.L * p.Hq; k += 32)
     reinterpret_cast<float*>(p.counts)[k] = static_cast<float>(static_cast<double>(__ldcg(p.counts + k)) / p.pairs);
