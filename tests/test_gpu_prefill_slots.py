@@ -1,5 +1,5 @@
-"""The attention kernel's two tile slots at the sizes where they can go wrong: fewer tiles than SMs and more than two per
-SM, tiles of one step, unions of an odd number of blocks of 64, rows that select nothing between rows that do, steps whose
+"""The attention kernel's two tile slots at the sizes where they can go wrong: fewer tiles than SMs, more than two per SM and
+more than three per slot (empty ones between others), tiles of one step, unions of an odd number of blocks of 64, rows that select nothing between rows that do, steps whose
 two key blocks belong to different rows, and the mask row of the first head of a pair under group-shared masks.
 
 The bound: bf16 inputs and outputs, probabilities rounded to bf16 (2^-9 relative each) before fp32 accumulation; against
@@ -30,7 +30,10 @@ def _reference(q, k, v, keep, block):
     (1024, 64, 2, 2, "apart"),         # neighbouring rows select different blocks
     (1024, 128, 4, 2, "empty"),        # empty rows between others
     (1000, 256, 2, 1, "random"),       # a block whose second sub-block is short
-    (1408, 128, 32, 4, "diagonal"),    # 352 tiles of one step: every slot takes several
+    (1408, 128, 32, 4, "diagonal"),    # 352 tiles of one step, more than the 296 slots of 148 SMs
+    (3840, 128, 32, 4, "alternating"),  # 960 tiles, every second one empty: every slot takes three or more
+    (3840, 64, 32, 4, "alternating"),
+    (3800, 256, 32, 4, "diagonal"),
     (1408, 64, 32, 4, "empty"),
     (2304, 256, 16, 2, "random"),
 ])
@@ -47,6 +50,8 @@ def test_slots_against_64_bits(n, block, hq, hkv, pattern):
         keep[:] = i[None, :] % 2 == i[:, None] % 2
     elif pattern == "empty":
         keep[:, i % 3 != 0] = False
+    elif pattern == "alternating":      # whole tiles of 128 rows: two blocks of 64
+        keep[:] = (i[None, :] == i[:, None]) & (i[:, None] // (128 // block) % 2 == 1)
     elif pattern == "diagonal":
         keep[:] = i[None, :] == i[:, None]
     w = (m + 31) // 32
