@@ -256,10 +256,11 @@ RBS_API rbs_status rbs_mask_group_union(const rbs_shape* shape, int q_start_bloc
 
 /*
  * rbs_sparse_prefill for group-shared masks: the caller states that the G query heads of every KV group have identical
- * mask rows (as rbs_mask_group_union leaves them).  The heads of a group run next to each other, so that the K/V tiles they have in common
- * come from L2; results are those of rbs_sparse_prefill bit for bit.  The paper's selector is per query head (Sec. 3.2), so this execution variant has no counterpart there; the attention it
- * computes is Sec. 3.3's.  Arguments and outputs as rbs_sparse_prefill (whole sequence only, no workspace); the mask is
- * read from the first head of each pair.  Needs block >= 128 and an even group size (RBS_ERR_UNSUPPORTED otherwise)
+ * mask rows (as rbs_mask_group_union leaves them).  The heads of a group run next to each other, so that the K/V tiles
+ * they have in common come from L2; results are those of rbs_sparse_prefill bit for bit.  The paper's selector is per
+ * query head (Sec. 3.2), so this execution variant has no counterpart there; the attention it computes is Sec. 3.3's.
+ * Arguments and outputs as rbs_sparse_prefill (whole sequence only, no workspace); the mask is read from the first head
+ * of each pair.  Needs block >= 128 and an even group size (RBS_ERR_UNSUPPORTED otherwise)
  * and a mask (RBS_ERR_INVALID_ARG for NULL).
  */
 RBS_API rbs_status rbs_sparse_prefill_grouped(const rbs_shape* shape, rbs_tensor Q, rbs_tensor K, rbs_tensor V,

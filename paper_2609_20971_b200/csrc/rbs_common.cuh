@@ -42,7 +42,9 @@ rbs_status check_chunk(const Dims& x, int q_start_block, int n_q_tokens);
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Workspace carve-up of rbs_select (all offsets 256-byte aligned).
+// Workspace carve-up of rbs_select (all offsets 256-byte aligned).  off_counts: one word, the CTAs of the scoring kernel that
+// have finished (the kept pairs are counted in the caller's density array); its space is that of L * Hq words, as it was
+// when the counts stood there, so that sizes callers have stored stay right.
 struct SelectWorkspace {
   size_t off_chi, off_clo, off_g, off_cn, off_perm, off_counts, bytes;
   int Mpad;  // centroid rows per (l, hk) in the bf16 copies, multiple of 128
@@ -166,9 +168,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src));
-}
 // 16-byte copy that writes zeros instead when `valid` is false (nothing is read from `src` then)
 __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, bool valid) {
   const uint32_t n = valid ? 16u : 0u;
