@@ -36,8 +36,6 @@ NCU_TRAFFIC_BYTES = {
 NOMINAL_BF16_TFLOPS = 2250.0     # dense bf16 per B200, for context next to the measured peak
 TARGET_TENSOR_FRAC = 0.60        # select + sparse attention on the selected FLOPs, of the measured bf16 peak
 TARGET_HBM_FRAC = 0.70           # statistics pass, of the measured copy bandwidth
-# kernels per step of the path: block_stats; select_prep, select_pair, density; prefill_duo
-LAUNCHES_PER_STEP = 5
 # the bounded oracle sample both arms time (the same in `cpu_baseline` and in `--impl reference`)
 ORACLE_SAMPLE = dict(n_heads=4, n_att_rows=48)
 
@@ -63,6 +61,43 @@ def config_dict(cfg) -> dict:
     """The `config` object of the JSON line (identical in both arms)."""
     return {"workload": cfg.name, "l2": "inputs larger than L2 (Q + O of one layer are 2 GiB or more); no flush",
             **cfg.describe()}
+
+
+def launches_per_step(cfg) -> int:
+    """Kernels per step of the path: block_stats; select_prep, the scoring kernel and, in all but short calls, density;
+    prefill_duo."""
+    import ctypes
+    from paper_2609_20971_b200.binding import RbsShape, load_library
+    shape = RbsShape(cfg.L, cfg.N, cfg.Hq, cfg.Hkv, cfg.d, cfg.B)
+    return 2 + load_library().rbs_selftest_select_launches(ctypes.byref(shape), cfg.N)
+
+
+def time_host_copies(hp, Qh, Kh, Vh, Oh, reps: int) -> float:
+    """ms per step of the end-to-end call's copies alone: the same pieces on the same two streams, without the kernels."""
+    main = torch.cuda.current_stream()
+
+    def copies():
+        hp.s_in.wait_stream(main)
+        hp.s_out.wait_stream(main)
+        with torch.cuda.stream(hp.s_in):
+            hp.Kg.copy_(Kh, non_blocking=True)
+            hp.Vg.copy_(Vh, non_blocking=True)
+            for _, _, _, t0, t1 in hp.chunks():
+                hp.Qg[:, t0:t1].copy_(Qh[:, t0:t1], non_blocking=True)
+        with torch.cuda.stream(hp.s_out):
+            for _, _, _, t0, t1 in hp.chunks():
+                Oh[:, t0:t1].copy_(hp.Og[:, t0:t1], non_blocking=True)
+        main.wait_stream(hp.s_in)
+        main.wait_stream(hp.s_out)
+    copies()
+    torch.cuda.synchronize()
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    e0.record(main)
+    for _ in range(reps):
+        copies()
+    e1.record(main)
+    torch.cuda.synchronize()
+    return e0.elapsed_time(e1) / reps
 
 
 def useful_flops(dens: np.ndarray, L: int, Hq: int, M: int, B: int, d: int):
@@ -432,7 +467,9 @@ def run_ours(args):
     barrier()
     e2e_ms = e0.elapsed_time(e1) / n_e2e
     e2e_ms = max_over_ranks(e2e_ms, world, dev)
-    e2e_launches = (1 + sum(1 for _ in hp.chunks()) * 5) * n_e2e
+    # the host link's share of it (it differs from box to box): the same copies without the kernels
+    copies_ms = time_host_copies(hp, Qh, Kh, Vh, Oh, n_e2e)
+    barrier()
     del hp
     h2d = Qh.numel() * 2 + Kh.numel() * 2 + Vh.numel() * 2
     d2h = Oh.numel() * 2
@@ -465,22 +502,21 @@ def run_ours(args):
             torch.cuda.synchronize()
             chunk[f"last_64_query_blocks_ms_{name}"] = e0.elapsed_time(e1) / 3
 
-    # group-shared masks (union over the G heads of a KV group): the one-head-per-CTA kernel on the union mask against
-    # the head-packed kernel (two heads per CTA over one K/V stream)
+    # group-shared masks (union over the G heads of a KV group): the two entry points on the union mask (one kernel)
     grouped = {}
     if rank == 0 and B >= 128 and (cfg.Hq // cfg.Hkv) % 2 == 0 and args.detail == "full":
         from paper_2609_20971_b200 import rbs_mask_group_union, rbs_sparse_prefill_grouped
         mu, du = mask.clone(), density.clone()
         rbs_mask_group_union(mu, du, cfg.Hkv, B, cfg.N)
-        for name, fn in (("one_head_per_cta", lambda: rbs_sparse_prefill(Qg, Kg, Vg, mu, B, out=Og)),
-                         ("two_heads_per_cta", lambda: rbs_sparse_prefill_grouped(Qg, Kg, Vg, mu, B, out=Og))):
+        for name, fn in (("sparse_prefill", lambda: rbs_sparse_prefill(Qg, Kg, Vg, mu, B, out=Og)),
+                         ("sparse_prefill_grouped", lambda: rbs_sparse_prefill_grouped(Qg, Kg, Vg, mu, B, out=Og))):
             fn()
             torch.cuda.synchronize()
             e0.record(stream)
             fn()
             e1.record(stream)
             torch.cuda.synchronize()
-            grouped[f"t_sparse_ms_{name}"] = e0.elapsed_time(e1)
+            grouped[f"t_ms_{name}"] = e0.elapsed_time(e1)
         grouped["density_of_union"] = float(du.float().mean().item())
         del mu, du
 
@@ -575,7 +611,7 @@ def run_ours(args):
         "cpu_baseline": ({"value": cpu_ms, "unit": UNIT, "cores": torch.get_num_threads(), "kind": "oracle",
                           "sample": cpu_sample, "parts": cpu_parts} if cpu_ms is not None else None),
         "e2e": {"value": ms_per_layer(e2e_ms, world, L), "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": LAUNCHES_PER_STEP * args.steps,
+        "gpu_launches": launches_per_step(cfg) * args.steps,
         "clocks": clocks,
         "detail": {
             "t_stats_ms": t_stats, "t_select_ms": t_select, "t_sparse_ms": t_sparse, "t_dense_ms": t_dense,
@@ -583,6 +619,7 @@ def run_ours(args):
             "speedup_vs_dense_incl_stats": t_dense / (t_stats + t_select + t_sparse),
             "density_mean": float(dens.mean()), "density_min": float(dens.min()), "density_max": float(dens.max()),
             "selected_tflop_useful": useful / 1e12,
+            "e2e_copies_alone_ms": ms_per_layer(copies_ms, world, L),
             "tensor_frac_select_plus_sparse": target_frac,
             "dense_tflops": dense_useful / (t_dense * 1e-3) / 1e12,
             "dense_tensor_frac": dense_useful / (t_dense * 1e-3) / 1e12 / peaks["tflops"],
