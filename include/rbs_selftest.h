@@ -65,6 +65,13 @@ RBS_API rbs_status rbs_selftest_debug_check(unsigned int* skipped, void* stream)
  */
 RBS_API rbs_status rbs_selftest_attention_wait(int warp, int which, int before);
 
+/*
+ * Debug build only: the same for the selections that follow: epilogue warp `warp` (0 .. 15; negative: none any more) of the
+ * two-head scoring kernel does its wait for an accumulator that has `before` such waits in front of it on a barrier that
+ * nothing arrives on, with 64 probes.
+ */
+RBS_API rbs_status rbs_selftest_select_wait(int warp, int before);
+
 #ifdef __cplusplus
 }
 #endif

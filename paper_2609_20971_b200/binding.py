@@ -100,6 +100,8 @@ def load_library() -> ctypes.CDLL:
     lib.rbs_selftest_warp_wait.argtypes = [vp, vp]
     lib.rbs_selftest_attention_wait.restype = i
     lib.rbs_selftest_attention_wait.argtypes = [i, i, i]
+    lib.rbs_selftest_select_wait.restype = i
+    lib.rbs_selftest_select_wait.argtypes = [i, i]
     lib.rbs_selftest_debug_check.restype = i
     lib.rbs_selftest_debug_check.argtypes = [vp, vp]
     lib.rbs_status_string.restype = ctypes.c_char_p
@@ -205,6 +207,15 @@ def rbs_selftest_attention_wait(warp: int, which: int = 0, before: int = 0) -> b
     if rc == 2:       # RBS_ERR_UNSUPPORTED: release build
         return False
     _check(rc, "rbs_selftest_attention_wait")
+    return True
+
+
+def rbs_selftest_select_wait(warp: int, before: int = 0) -> bool:
+    """Debug library only: the same for one epilogue warp of the two-head scoring kernel in the selections that follow."""
+    rc = load_library().rbs_selftest_select_wait(warp, before)
+    if rc == 2:       # RBS_ERR_UNSUPPORTED: release build
+        return False
+    _check(rc, "rbs_selftest_select_wait")
     return True
 
 

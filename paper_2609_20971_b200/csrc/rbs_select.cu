@@ -380,6 +380,11 @@ constexpr int kPairProducer = 16, kPairMma = 17;
 // group to the first like the token halves inside a group; the first group alone keeps the scores and writes the mask.
 // ODD: the group size is odd (a kernel of its own: as a run-time flag it cost the other group sizes 3 %).
 // FINISH: the last CTA turns the counts into densities instead of density_kernel (see finishes_itself).
+#ifdef RBS_DEBUG
+// rbs_selftest_select_wait: {epilogue warp (-1: none), how many of its waits for an accumulator come before}: that wait is
+// done on a barrier that nothing arrives on, with 64 probes.
+static __device__ int g_selftest_select[2] = {-1, 0};
+#endif
 template <int B, bool HALVES, bool ODD, bool FINISH>
 __global__ void __launch_bounds__(kPairThreads, 1)
 select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmChi,
@@ -404,6 +409,9 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __shared__ __align__(8) float2 sGroup[4][2][32];
   __shared__ float sRed[2][2][8], sRedQ[2][16], sQstat[2][2];
   __shared__ uint32_t s_tmem;
+#ifdef RBS_DEBUG
+  __shared__ __align__(8) uint64_t bar_never;
+#endif
 
   const int tid = threadIdx.x, lane = tid & 31;
   // The warp index from a shuffle is uniform for the compiler, so that the roles run on uniform branches and registers
@@ -431,6 +439,9 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       }
       for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&bar_group[q][s]), 1);
     }
+#ifdef RBS_DEBUG
+    mbar_init(smem_u32(&bar_never), 1);
+#endif
     mbar_fence_init();
   }
   if (warp == kPairMma) tmem_alloc(smem_u32(&s_tmem), 4 * B);
@@ -569,7 +580,19 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     float* sLr = sLb + l_floats;
     uint32_t nt = 0, k = 0;
     bool ok = true;
-    for (int w = valid(blockIdx.x); ok && w < n_items; w = valid(w + gridDim.x), ++k) {
+#ifdef RBS_DEBUG
+    int st_before = g_selftest_select[1];
+#endif
+    auto wait_accumulator = [&](uint64_t* bar, uint32_t parity) -> bool {
+#ifdef RBS_DEBUG
+      if (g_selftest_select[0] == warp && st_before-- == 0)
+        return mbar_wait_limit(smem_u32(&bar_never), 0, status, kWaitSelfTest, 64);
+#endif
+      return mbar_wait(smem_u32(bar), parity, status, kWaitMmaDone);
+    };
+    // (HALVES: a group whose wait gave up inside an item stays until the barrier of both groups in the next one, behind which
+    // both leave: the other group would wait there for ever)
+    for (int w = valid(blockIdx.x); (HALVES || ok) && w < n_items; w = valid(w + gridDim.x), ++k) {
       const Item it = decode(w);
       const int l = it.l, hk = it.hk, h = hw == 0 ? it.h0 : it.h1;
       const bool real = !ODD || hw == 0 || it.il1 >= 0;         // a half that does not exist repeats the first one and writes nothing
@@ -579,7 +602,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int crow0 = static_cast<int>((static_cast<int64_t>(l) * Hkv + hk) * p.Mpad);
       const uint32_t slot = k & 1;
       const unsigned char* q = sQ + slot * 2 * kQTile + hw * kPanelQ;
-      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_qfull[slot]), (k >> 1) & 1, status, kWaitTmaFull));
+      ok = __all_sync(0xffffffffu, (!HALVES || ok) && mbar_wait(smem_u32(&bar_qfull[slot]), (k >> 1) & 1, status, kWaitTmaFull));
       const int n_tok = HALVES ? max(0, min(B, p.Nq - il * QB - hw * B)) : min(B, p.Nq - il * B);   // of this group
       float qn_max, qn_spread;
       ok = query_norm_shifts<B, 256, kQTile>(q, wtid, n_tok, sQn_h, &sRedQ[hw][0], gbar, ok, qn_max, qn_spread);
@@ -588,11 +611,12 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // the norms' maximum and spread are those of the whole block of 2 B tokens: exchange with the other group
         if (wtid == 0) { sQstat[hw][0] = qn_max; sQstat[hw][1] = n_tok > 0 ? qn_max - qn_spread : INFINITY; }
         ok = group_all<512>(ok, 3);                                  // both groups (and a failed wait ends both)
+        if (!ok) break;
         const float g_max = fmaxf(sQstat[0][0], sQstat[1][0]), g_min = fminf(sQstat[0][1], sQstat[1][1]);
         if (wtid < B) sQn_h[wtid] -= g_max - qn_max;                // shifts relative to the block's maximum
         qn_max = g_max;
         qn_spread = g_max - g_min;
-        ok = group_all<512>(ok, 3);                                  // shifts written; sQstat may be rewritten by the next item
+        (void)group_all<512>(true, 3);                               // shifts written; sQstat may be rewritten by the next item
       }
       float mxb = -INFINITY, mxr = -INFINITY;     // running maxima of this thread's L values (causal blocks only)
       for (int bt = 0; ok && bt < n_tiles; ++bt, ++nt) {
@@ -602,7 +626,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const bool prow_ok = RBS_DBG_OK(prow >= 0 && prow < p.L * Hkv * p.Mpad, status, kDbgSelectCentroid);
         const float gs = prow_ok ? __ldg(p.gs + prow) : 0.f, cn = prow_ok ? __ldg(p.cnorm + prow) : 0.f;
         const int b_row = prow_ok ? __ldg(p.perm + prow) : 0x7fffffff;   // the block this accumulator row belongs to
-        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_tfull[hw][buf]), (nt >> 1) & 1, status, kWaitMmaDone));
+        ok = __all_sync(0xffffffffu, wait_accumulator(&bar_tfull[hw][buf], (nt >> 1) & 1));
         if (!ok) break;
         tc_fence_after_sync();
         (void)RBS_DBG_OK(acc_col(hw, buf) + B <= 4u * B, status, kDbgSelectTmem);
@@ -907,6 +931,18 @@ extern "C" rbs_status rbs_select_variant(const rbs_shape* shape, rbs_tensor Q, r
                          dbg_base_mask, dbg_rescue_mask, workspace, workspace_bytes, stream);
   }
   return RBS_ERR_INVALID_ARG;
+}
+
+extern "C" rbs_status rbs_selftest_select_wait(int warp, int before) {
+#ifdef RBS_DEBUG
+  if (warp > 15 || before < 0) return RBS_ERR_INVALID_ARG;
+  const int v[2] = {warp < 0 ? -1 : warp, before};
+  RBS_CUDA_OK(cudaMemcpyToSymbol(rbs::g_selftest_select, v, sizeof(v)));
+  return RBS_OK;
+#else
+  (void)warp; (void)before;
+  return RBS_ERR_UNSUPPORTED;   // the release build has no such switch
+#endif
 }
 
 extern "C" int rbs_selftest_select_launches(const rbs_shape* shape, int n_q_tokens) {

@@ -148,3 +148,45 @@ def test_a_softmax_warp_whose_wait_runs_out_takes_the_launch_to_its_end():
     r = subprocess.run([sys.executable, "-c", WAIT_CHILD, repr(WAITS)], env=env, cwd=ROOT, capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0 and "wait child ok" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+SELECT_WAIT_CHILD = r"""
+import sys, time, torch
+from paper_2609_20971_b200 import rbs_block_stats, rbs_select, rbs_device_status
+from paper_2609_20971_b200.binding import rbs_selftest_select_wait
+N, Hq, Hkv = 256 * 140 - 70, 4, 2          # 560 items at blocks of 256: three or four per CTA, one or two tiles each
+g = torch.Generator(device="cuda").manual_seed(6)
+Q, K = (torch.randn(1, N, h, 128, generator=g, device="cuda").bfloat16() for h in (Hq, Hkv))
+stats = {B: rbs_block_stats(K, B) for B in (128, 256)}
+want = {B: rbs_select(Q, stats[B], B) for B in stats}
+assert rbs_device_status(clear=True) == 0
+for B, warp, before in eval(sys.argv[1]):
+    assert rbs_selftest_select_wait(warp, before)
+    t = time.time()
+    rbs_select(Q, stats[B], B)
+    torch.cuda.synchronize()
+    t = time.time() - t
+    code = rbs_device_status(clear=True)
+    assert rbs_selftest_select_wait(-1)
+    print("case", B, warp, before, "%.3f s" % t, flush=True)
+    assert code == 7 and t < 20.0, code
+    for b in want:
+        assert all(torch.equal(x, y) for x, y in zip(rbs_select(Q, stats[b], b), want[b]))
+    assert rbs_device_status(clear=True) == 0
+print("select wait child ok")
+"""
+
+
+def test_an_epilogue_warp_whose_wait_runs_out_takes_the_selection_to_its_end():
+    """The same for the two-head scoring kernel.  At blocks of 256 its two epilogue groups meet at a barrier in every item: a
+    group whose wait ran out must not leave the other one there."""
+    from paper_2609_20971_b200.binding import rbs_selftest_select_wait
+    from paper_2609_20971_b200.build import build_library
+    assert rbs_selftest_select_wait(0) is False
+    build_library(debug=True)
+    env = dict(os.environ, RBS_DEBUG="1", PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    # (block, warp, waits before): both groups, both token halves, first and later items
+    waits = [(B, warp, before) for B in (128, 256) for warp, before in ((3, 0), (5, 3), (9, 1), (12, 0), (14, 4))]
+    r = subprocess.run([sys.executable, "-c", SELECT_WAIT_CHILD, repr(waits)], env=env, cwd=ROOT, capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and "select wait child ok" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
