@@ -548,9 +548,8 @@ def test_long_rows_are_split_and_merged(B, M, tail):
 
 
 def test_grouped_attention_under_group_shared_masks():
-    """Head-packed query tiles: with the masks of a KV group made identical (rbs_mask_group_union) two heads of the group
-    share one stream of K/V tiles.  Against the oracle (attention over the oracle's union of the GPU's per-head masks) and
-    against the one-head-per-CTA kernel on the same mask."""
+    """Attention under group-shared masks (made identical inside every KV group by rbs_mask_group_union), against the oracle
+    (attention over the oracle's union of the GPU's per-head masks) and against rbs_sparse_prefill on the same mask."""
     from paper_2609_20971_b200 import rbs_sparse_prefill_grouped
     for cfg in (SynthConfig("grouped", L=2, N=128 * 45 + 50, Hq=8, Hkv=2, B=128, sigma=(0.1, 1.0), seed=62),
                 SynthConfig("grouped256", N=256 * 21, Hq=4, Hkv=2, B=256, sigma=0.6, seed=63)):
