@@ -590,9 +590,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #endif
       return mbar_wait(smem_u32(bar), parity, status, kWaitMmaDone);
     };
-    // (HALVES: a group whose wait gave up inside an item stays until the barrier of both groups in the next one, behind which
-    // both leave: the other group would wait there for ever)
-    for (int w = valid(blockIdx.x); (HALVES || ok) && w < n_items; w = valid(w + gridDim.x), ++k) {
+    for (int w = valid(blockIdx.x); ok && w < n_items; w = valid(w + gridDim.x), ++k) {
       const Item it = decode(w);
       const int l = it.l, hk = it.hk, h = hw == 0 ? it.h0 : it.h1;
       const bool real = !ODD || hw == 0 || it.il1 >= 0;         // a half that does not exist repeats the first one and writes nothing
@@ -602,7 +600,7 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int crow0 = static_cast<int>((static_cast<int64_t>(l) * Hkv + hk) * p.Mpad);
       const uint32_t slot = k & 1;
       const unsigned char* q = sQ + slot * 2 * kQTile + hw * kPanelQ;
-      ok = __all_sync(0xffffffffu, (!HALVES || ok) && mbar_wait(smem_u32(&bar_qfull[slot]), (k >> 1) & 1, status, kWaitTmaFull));
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_qfull[slot]), (k >> 1) & 1, status, kWaitTmaFull));
       const int n_tok = HALVES ? max(0, min(B, p.Nq - il * QB - hw * B)) : min(B, p.Nq - il * B);   // of this group
       float qn_max, qn_spread;
       ok = query_norm_shifts<B, 256, kQTile>(q, wtid, n_tok, sQn_h, &sRedQ[hw][0], gbar, ok, qn_max, qn_spread);
@@ -610,13 +608,12 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       if (HALVES) {
         // the norms' maximum and spread are those of the whole block of 2 B tokens: exchange with the other group
         if (wtid == 0) { sQstat[hw][0] = qn_max; sQstat[hw][1] = n_tok > 0 ? qn_max - qn_spread : INFINITY; }
-        ok = group_all<512>(ok, 3);                                  // both groups (and a failed wait ends both)
-        if (!ok) break;
+        ok = group_all<512>(ok, 3);                                  // both groups
         const float g_max = fmaxf(sQstat[0][0], sQstat[1][0]), g_min = fminf(sQstat[0][1], sQstat[1][1]);
         if (wtid < B) sQn_h[wtid] -= g_max - qn_max;                // shifts relative to the block's maximum
         qn_max = g_max;
         qn_spread = g_max - g_min;
-        (void)group_all<512>(true, 3);                               // shifts written; sQstat may be rewritten by the next item
+        ok = group_all<512>(ok, 3);                                  // shifts written; sQstat may be rewritten by the next item
       }
       float mxb = -INFINITY, mxr = -INFINITY;     // running maxima of this thread's L values (causal blocks only)
       for (int bt = 0; ok && bt < n_tiles; ++bt, ++nt) {
@@ -699,6 +696,10 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           mxr = fmaxf(mxr, Lr);
         }
       }
+      // HALVES: the first group reads the second one's norms where it takes exact shifts, so the second group, which has nothing
+      // to do in such tiles, may not begin the next item before the first one is through its tiles; and a failed wait ends
+      // both groups here, since either would wait for the other one in the next item.
+      if (HALVES) ok = group_all<512>(ok, 3);
       // row maxima over the causal candidates, thresholds, forced blocks, union, pack: this group alone
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {

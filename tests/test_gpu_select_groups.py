@@ -65,3 +65,23 @@ def test_odd_groups_against_the_oracle(L, Hq, Hkv, B, N, launches, chunks):
         pairs = sum(i + 1 for i in range(q0, q1))
         assert np.array_equal(dc.cpu().numpy(), (final[:, :, q0:q1].sum((2, 3)) / pairs).astype(np.float32))
     assert rbs_device_status(clear=True) == 0
+
+
+@pytest.mark.parametrize("L, Hq, Hkv, N", [(3, 3, 3, 35585), (1, 16, 2, 256 * 60 + 9)])
+def test_blocks_of_256_with_exact_shifts(L, Hq, Hkv, N):
+    """Keys whose norms grow over the sequence take most rows past the range of the norm bounds, where one of the two epilogue
+    groups of a block of 256 takes the exact maxima of both halves alone and the other one has nothing to do.  A call of many
+    items per thread block must give the bits of chunked calls in which no thread block has a second item."""
+    B = 256
+    M = (N + B - 1) // B
+    g = torch.Generator(device="cuda").manual_seed(N)
+    Q, K = (torch.randn(L, N, h, 128, generator=g, device="cuda") for h in (Hq, Hkv))
+    K *= (1 + torch.arange(N, device="cuda") / 200.0).view(1, N, 1, 1)
+    Q, K = (3 * Q).bfloat16(), K.bfloat16()
+    stats = rbs_block_stats(K, B)
+    rows = max(1, 100 // (L * Hq))                      # items per chunked call: at most 100, one per thread block
+    want = torch.cat([rbs_select_chunk(Q[:, q0 * B:min(N, (q0 + rows) * B)], stats, B, N, q0)[0] for q0 in range(0, M, rows)], dim=2)
+    for _ in range(20):
+        mask, _ = rbs_select(Q, stats, B)
+        assert torch.equal(mask, want)
+    assert rbs_device_status(clear=True) == 0
