@@ -204,33 +204,48 @@ prefill_mma_kernel(const PrefillParams p) {
 // ---------------------------------------------------------------------------------------------
 constexpr int kPlanThreads = 1024;
 
-// number of 128-key sub-blocks tile T of query block i attends in mask row `row`: R per selected block below the
-// diagonal block, and the diagonal block's sub-blocks up to T
-__device__ __forceinline__ int count_kb_fast(const uint32_t* __restrict__ row, int i, int R, int T) {
-  int n = 0;
-  const int wi = i >> 5;
-  for (int w = 0; w < wi; ++w) n += __popc(__ldg(row + w));
-  const uint32_t u = __ldg(row + wi) & (0xffffffffu >> (31 - (i & 31)));
-  const uint32_t diag = (u >> (i & 31)) & 1u;
-  return R * (n + __popc(u) - static_cast<int>(diag)) + (diag ? T - i * R + 1 : 0);
+// Sub-blocks of 128 keys that word w of a mask row stands for: R per selected block before query block i, and of block i
+// itself those up to tile T.  u: the word's causal bits.
+__device__ __forceinline__ int word_kb(uint32_t u, int w, int i, int R, int T) {
+  const bool diag = w == (i >> 5) && ((u >> (i & 31)) & 1u);
+  return R * __popc(u) - (diag ? R - (T - i * R + 1) : 0);
+}
+__device__ __forceinline__ uint32_t causal_word(const uint32_t* __restrict__ row, int w, int i) {
+  const uint32_t u = w <= (i >> 5) ? __ldg(row + w) : 0u;
+  return w == (i >> 5) ? u & (0xffffffffu >> (31 - (i & 31))) : u;
 }
 
-// the same count by walking the set bits, stopping at ordinal `stop` (>= 0): *kb_at receives the index of the
-// sub-block with that ordinal
-__device__ __forceinline__ int count_kb(const uint32_t* __restrict__ row, int i, int R, int T, int stop, int* kb_at) {
-  int n = 0;
-  for (int w = 0; w <= (i >> 5); ++w) {
-    uint32_t u = __ldg(row + w);
-    if (((w + 1) << 5) - 1 > i) u &= 0xffffffffu >> (31 - (i & 31));
-    while (u) {
-      const int b = (w << 5) + __ffs(u) - 1;
-      u &= u - 1;
-      const int first = b * R, last = min(b * R + R - 1, T);   // this block's sub-blocks up to the diagonal
-      if (stop >= 0 && n + (last - first + 1) > stop) { *kb_at = first + (stop - n); return stop; }
-      n += last - first + 1;
+// The index of the sub-block with ordinal `stop` in a row that has more than `stop` of them; a converged warp, a lane per
+// word.
+__device__ __forceinline__ int kb_at_ordinal(const uint32_t* __restrict__ row, int i, int R, int T, int stop) {
+  const int lane = threadIdx.x & 31;
+  for (int w0 = 0; w0 <= (i >> 5); w0 += 32) {
+    const int w = w0 + lane;
+    uint32_t u = causal_word(row, w, i);
+    const int n = word_kb(u, w, i, R, T);
+    int upto = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
     }
+    const uint32_t past = __ballot_sync(0xffffffffu, upto > stop);
+    if (past == 0u) { stop -= __shfl_sync(0xffffffffu, upto, 31); continue; }
+    int kb = 0;
+    const int src = __ffs(past) - 1;
+    if (lane == src) {
+      int before = upto - n;
+      while (u) {
+        const int b = (w << 5) + __ffs(u) - 1;
+        u &= u - 1;
+        const int first = b * R, last = min(b * R + R - 1, T);   // this block's sub-blocks up to the diagonal
+        if (before + (last - first + 1) > stop) { kb = first + (stop - before); break; }
+        before += last - first + 1;
+      }
+    }
+    return __shfl_sync(0xffffffffu, kb, src);
   }
-  return n;
+  return 0;
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
@@ -238,6 +253,8 @@ plan_rows_kernel(const PrefillParams p, int4* __restrict__ items, int4* __restri
   extern __shared__ int s_cnt[];                     // sub-blocks per row of the group, in static order
   __shared__ int s_warp_long[kPlanThreads / 32];
   __shared__ int s_split_pos[kSplitRowsPerGroup], s_split_parts[kSplitRowsPerGroup], s_n_split;
+  pdl_wait();
+  pdl_trigger();
   const int R = p.R, Hkv = p.Hq / p.G;
   const int n_g = p.band_rows * p.G;               // rows (128-row tiles) per group
   const int g = blockIdx.x;                        // band * (L * Hkv) + kvid
@@ -253,17 +270,38 @@ plan_rows_kernel(const PrefillParams p, int4* __restrict__ items, int4* __restri
     row = p.mask + ((static_cast<int64_t>(l) * p.Hq + h) * p.Mq + (i - p.q0)) * p.W;
     return true;
   };
+  // a warp counts four rows at a time, a lane per word
+  constexpr int kWarps = kPlanThreads / 32, kAtOnce = 4;
+  for (int p0 = warp; p0 < n_g; p0 += kWarps * kAtOnce) {
+    int cnt[kAtOnce], T[kAtOnce], i[kAtOnce];
+    const uint32_t* row[kAtOnce];
+    bool there[kAtOnce];
+    int i_max = -1;
+#pragma unroll
+    for (int u = 0; u < kAtOnce; ++u) {
+      int Tl;
+      cnt[u] = 0;
+      i[u] = -1;
+      there[u] = p0 + u * kWarps < n_g && tile_of(p0 + u * kWarps, Tl, T[u], i[u], row[u]);
+      if (there[u]) i_max = max(i_max, i[u]);
+    }
+    for (int w = lane; w <= (i_max >> 5); w += 32) {
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u)
+        if (there[u]) cnt[u] += word_kb(causal_word(row[u], w, i[u]), w, i[u], R, T[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kAtOnce; ++u) {
+      const int sum = __reduce_add_sync(0xffffffffu, cnt[u]);
+      if (lane == 0 && p0 + u * kWarps < n_g) s_cnt[p0 + u * kWarps] = there[u] ? sum : -1;   // -1: no such tile
+    }
+  }
+  __syncthreads();
   // every thread owns a contiguous run of rows, so that ranks in static order come from one scan over the threads
   const int per_thread = (n_g + kPlanThreads - 1) / kPlanThreads;
   const int first = tid * per_thread, last = min(n_g, first + per_thread);
   int n_long = 0;
-  for (int pos = first; pos < last; ++pos) {
-    int Tl, T, i;
-    const uint32_t* row;
-    const int cnt = tile_of(pos, Tl, T, i, row) ? count_kb_fast(row, i, R, T) : -1;   // -1: no such tile
-    s_cnt[pos] = cnt;
-    n_long += cnt > kSplitCap;
-  }
+  for (int pos = first; pos < last; ++pos) n_long += s_cnt[pos] > kSplitCap;
   if (tid == 0) s_n_split = 0;
   // exclusive scan of n_long over the threads
   int incl = n_long;
@@ -302,35 +340,39 @@ plan_rows_kernel(const PrefillParams p, int4* __restrict__ items, int4* __restri
     if (!is_split) out[at] = s_cnt[pos] >= 0 ? make_int4(pos, 0, 0x7fffffff, -1) : make_int4(-1, 0, 0, -1);
   }
   for (int e = n_g + extra_total + tid; e < per_group; e += kPlanThreads) out[e] = make_int4(-1, 0, 0, -1);   // unused
-  // the parts of the split rows: one thread per (row, part)
-  if (tid < kSplitRowsPerGroup * kSplitMaxParts) {
-    const int s = tid / kSplitMaxParts, part = tid % kSplitMaxParts;
-    if (s < n_split) {
-      const int pos = s_split_pos[s], parts = s_split_parts[s], cnt = s_cnt[pos];
-      if (part < parts) {
-        int at = pos + part;
-        for (int s2 = 0; s2 < s; ++s2) at += s_split_parts[s2] - 1;
-        int Tl, T, i;
-        const uint32_t* row;
-        tile_of(pos, Tl, T, i, row);
-        const int len = (cnt + parts - 1) / parts;
-        int kb_begin = 0, kb_end = T + 1;
-        if (part > 0) count_kb(row, i, R, T, part * len, &kb_begin);
-        if (part + 1 < parts) count_kb(row, i, R, T, (part + 1) * len, &kb_end);
-        out[at] = make_int4(pos, kb_begin, kb_end, g * kSplitSlotsPerGroup + s * kSplitMaxParts + part);
-      }
-      if (part == 0) splits[g * kSplitRowsPerGroup + s] = make_int4(pos, parts, 0, 0);
-    } else if (part == 0) {
-      splits[g * kSplitRowsPerGroup + s] = make_int4(-1, 1, 0, 0);
-    }
+  // the parts of the split rows: a warp per (row, part)
+  static_assert(kSplitRowsPerGroup * kSplitMaxParts == kWarps, "a warp per part");
+  const int s = warp / kSplitMaxParts, part = warp % kSplitMaxParts;
+  if (s >= n_split) {
+    if (part == 0 && lane == 0) splits[g * kSplitRowsPerGroup + s] = make_int4(-1, 1, 0, 0);
+    return;
   }
+  const int pos = s_split_pos[s], parts = s_split_parts[s], cnt = s_cnt[pos];
+  if (part < parts) {
+    int at = pos + part;
+    for (int s2 = 0; s2 < s; ++s2) at += s_split_parts[s2] - 1;
+    int Tl, T, i;
+    const uint32_t* row;
+    tile_of(pos, Tl, T, i, row);
+    const int len = (cnt + parts - 1) / parts;
+    const int kb_begin = part > 0 ? kb_at_ordinal(row, i, R, T, part * len) : 0;
+    const int kb_end = part + 1 < parts ? kb_at_ordinal(row, i, R, T, (part + 1) * len) : T + 1;
+    if (lane == 0) out[at] = make_int4(pos, kb_begin, kb_end, g * kSplitSlotsPerGroup + s * kSplitMaxParts + part);
+  }
+  if (part == 0 && lane == 0) splits[g * kSplitRowsPerGroup + s] = make_int4(pos, parts, 0, 0);
 }
 
 // Merges the parts of one split row: with m = max_p m_p,  l = sum_p l_p 2^(m_p - m),  O = sum_p O_p 2^(m_p - m) / l
 // (the maximum is only a shift, Sec. 3.3's softmax over the retained keys is unchanged), parts taken in order.
-// One CTA per (group, split-row slot), one thread per query row.
-__global__ void __launch_bounds__(128)
+// One CTA per (group, split-row slot, 16 query rows), a warp per row: bound by the latency of two dependent loads per row,
+// so that all of a CTA's rows are on their way together (the last 64 query blocks of 128K tokens of 32 heads, 32 split rows:
+// 69 us with 32 CTAs of four warps that take one row after the other; a whole pass over that chunk, with the warp-wide counting
+// of plan_rows_kernel, which took 135 us with a thread per row, 1,396 instead of 1,489 us).
+constexpr int kCombineRows = 16;
+__global__ void __launch_bounds__(kCombineRows * 32)
 combine_parts_kernel(const PrefillParams p, const int4* __restrict__ splits) {
+  pdl_wait();
+  pdl_trigger();
   const int4 sp = splits[blockIdx.x];
   if (sp.x < 0) return;
   const int g = blockIdx.x / kSplitRowsPerGroup, s = blockIdx.x % kSplitRowsPerGroup;
@@ -339,30 +381,40 @@ combine_parts_kernel(const PrefillParams p, const int4* __restrict__ splits) {
   const int l = kvid / Hkv, hk = kvid % Hkv;
   const int Tl = p.Mq * R - 1 - (band * p.band_rows + sp.x / p.G);
   const int h = hk * p.G + sp.x % p.G;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, row = blockIdx.y * kCombineRows + (threadIdx.x >> 5);
   const int slot0 = g * kSplitSlotsPerGroup + s * kSplitMaxParts;
-  // a warp takes one query row at a time, its lanes four output columns each (whole 512-byte lines per part)
-  for (int row = warp; row < 128; row += 4) {
-    if (Tl * 128 + row >= p.Nq) break;     // rows past the end of the queries are not written
-    float m = -INFINITY;
-    for (int q = 0; q < sp.y; ++q) m = fmaxf(m, p.part_ml[static_cast<int64_t>(slot0 + q) * 256 + row]);
-    float lsum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int q = 0; q < sp.y; ++q) {
-      const float* ml = p.part_ml + static_cast<int64_t>(slot0 + q) * 256;
-      const float w = fast_exp2(ml[row] - m);
-      lsum = fmaf(ml[128 + row], w, lsum);
-      const float4 a = *reinterpret_cast<const float4*>(p.part_o + (static_cast<int64_t>(slot0 + q) * 128 + row) * 128 + lane * 4);
-      acc.x = fmaf(a.x, w, acc.x); acc.y = fmaf(a.y, w, acc.y); acc.z = fmaf(a.z, w, acc.z); acc.w = fmaf(a.w, w, acc.w);
-    }
-    const float inv = 1.0f / lsum;
-    __nv_bfloat16* orow = p.O + l * p.osb + (static_cast<int64_t>(Tl) * 128 + row) * p.ost + h * p.osh;
-    uint2 v;
-    v.x = pack_bf16(acc.x * inv, acc.y * inv);
-    v.y = pack_bf16(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2*>(orow + lane * 4) = v;
-    if (p.lse && lane == 0) p.lse[(static_cast<int64_t>(l) * p.Hq + h) * p.Nq + Tl * 128 + row] = (m + fast_log2(lsum)) * 0.6931471805599453f;
+  if (Tl * 128 + row >= p.Nq) return;     // rows past the end of the queries are not written
+  // the lanes take four output columns each (whole 512-byte lines per part)
+  float mp[kSplitMaxParts], lp[kSplitMaxParts];
+  float4 a[kSplitMaxParts];
+#pragma unroll
+  for (int q = 0; q < kSplitMaxParts; ++q) {
+    if (q >= sp.y) continue;
+    const float* ml = p.part_ml + static_cast<int64_t>(slot0 + q) * 256;
+    mp[q] = ml[row];
+    lp[q] = ml[128 + row];
+    a[q] = *reinterpret_cast<const float4*>(p.part_o + (static_cast<int64_t>(slot0 + q) * 128 + row) * 128 + lane * 4);
   }
+  float m = -INFINITY;
+#pragma unroll
+  for (int q = 0; q < kSplitMaxParts; ++q)
+    if (q < sp.y) m = fmaxf(m, mp[q]);
+  float lsum = 0.f;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < kSplitMaxParts; ++q) {
+    if (q >= sp.y) continue;
+    const float w = fast_exp2(mp[q] - m);
+    lsum = fmaf(lp[q], w, lsum);
+    acc.x = fmaf(a[q].x, w, acc.x); acc.y = fmaf(a[q].y, w, acc.y); acc.z = fmaf(a[q].z, w, acc.z); acc.w = fmaf(a[q].w, w, acc.w);
+  }
+  const float inv = 1.0f / lsum;
+  __nv_bfloat16* orow = p.O + l * p.osb + (static_cast<int64_t>(Tl) * 128 + row) * p.ost + h * p.osh;
+  uint2 v;
+  v.x = pack_bf16(acc.x * inv, acc.y * inv);
+  v.y = pack_bf16(acc.z * inv, acc.w * inv);
+  *reinterpret_cast<uint2*>(orow + lane * 4) = v;
+  if (p.lse && lane == 0) p.lse[(static_cast<int64_t>(l) * p.Hq + h) * p.Nq + Tl * 128 + row] = (m + fast_log2(lsum)) * 0.6931471805599453f;
 }
 
 // Bands of the tile order.  Long sequences: up to four of at least 64 query tiles (512 tiles per band and KV head at
@@ -386,10 +438,11 @@ static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q,
   PrefillParams pp = p;
   const int n_rows = p.Mq * p.R;
   // the schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink
-  // steadily) and a group whose counts fit the planner's shared memory
+  // steadily), rows long enough to be cut (a row that is not cut gives the same bits either way; selection and attention of
+  // 2K of 8K tokens, 32 heads: 125 us without planner and merge, 153 with them) and a group whose counts fit the planner's shared memory
   const double kv_bytes = 4.0 * kHeadDim * p.L * Hkv * static_cast<double>(p.N);
   const int sched_bands = tile_bands(n_rows, true, 0.0);
-  const bool scheduled = p.mask != nullptr && workspace != nullptr &&
+  const bool scheduled = p.mask != nullptr && workspace != nullptr && (p.q0 + p.Mq) * p.R > kSplitCap &&
                          static_cast<size_t>((n_rows + sched_bands - 1) / sched_bands) * p.G * sizeof(int) <= 200 * 1024;
   const int n_bands = tile_bands(n_rows, scheduled, kv_bytes);
   pp.band_rows = (n_rows + n_bands - 1) / n_bands;
@@ -409,14 +462,12 @@ static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q,
     pp.part_o = reinterpret_cast<float*>(base + w.off_part_o);
     pp.part_ml = reinterpret_cast<float*>(base + w.off_part_ml);
     if ((st = ensure_dynamic_smem(reinterpret_cast<const void*>(plan_rows_kernel), plan_smem)) != RBS_OK) return st;
-    plan_rows_kernel<<<n_groups, kPlanThreads, plan_smem, s>>>(pp, items, splits);
-    RBS_CUDA_OK(cudaGetLastError());
+    RBS_CUDA_OK(launch_pdl(plan_rows_kernel, n_groups, 1, kPlanThreads, plan_smem, s, pp, items, splits));
   }
   const long long n_items = static_cast<long long>(n_groups) * (scheduled ? pp.items_per_group : rows_per_group);
   if ((st = launch_prefill_duo(pp, Q, K, V, Hkv, false, n_items, s)) != RBS_OK) return st;
   if (scheduled) {
-    combine_parts_kernel<<<n_groups * kSplitRowsPerGroup, 128, 0, s>>>(pp, splits);
-    RBS_CUDA_OK(cudaGetLastError());
+    RBS_CUDA_OK(launch_pdl(combine_parts_kernel, n_groups * kSplitRowsPerGroup, 128 / kCombineRows, kCombineRows * 32, 0, s, pp, splits));
   }
   return RBS_OK;
 }
