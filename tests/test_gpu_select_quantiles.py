@@ -16,7 +16,7 @@ def test_quantiles_of_radii(m):
     q = torch.randn(1, n, 4, 128, generator=g, device="cuda").bfloat16()
     stats = rbs_block_stats(k.bfloat16(), 64)
     r = stats.radius.view(hkv, m)
-    r[:, ::3] = r[:, :1]                    # ties
+    r[:, ::3] = r[:, :1].clone()                    # ties
     rbs_select(q, stats, 64)
     want = torch.quantile(r.double(), torch.tensor([0.5, 0.9], dtype=torch.float64, device="cuda"), dim=1).t()
     assert torch.allclose(stats.rq.view(hkv, 2).double(), want, rtol=2.0 ** -22, atol=0)
