@@ -132,7 +132,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KernelArgs...), unsigned grid_x, un
   if (e != cudaSuccess) (void)cudaGetLastError();
   return e;
 }
-// The kernels before this one in the stream have ended and their writes are visible.
+// The kernels before this one in the stream have ended and their writes are visible.  To plain loads, that is: a kernel
+// launched this way lives while its predecessor still writes, and the non-coherent path (__ldg, `const T* __restrict__`) is for
+// memory that nobody writes during the kernel's life; the compiler may also move such a load in front of this wait.  So
+// what another kernel of the path wrote (mask, items, statistics, scratch) is never read that way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

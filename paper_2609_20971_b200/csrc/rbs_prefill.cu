@@ -210,14 +210,14 @@ __device__ __forceinline__ int word_kb(uint32_t u, int w, int i, int R, int T) {
   const bool diag = w == (i >> 5) && ((u >> (i & 31)) & 1u);
   return R * __popc(u) - (diag ? R - (T - i * R + 1) : 0);
 }
-__device__ __forceinline__ uint32_t causal_word(const uint32_t* __restrict__ row, int w, int i) {
-  const uint32_t u = w <= (i >> 5) ? __ldg(row + w) : 0u;
+__device__ __forceinline__ uint32_t causal_word(const uint32_t* row, int w, int i) {
+  const uint32_t u = w <= (i >> 5) ? row[w] : 0u;
   return w == (i >> 5) ? u & (0xffffffffu >> (31 - (i & 31))) : u;
 }
 
 // The index of the sub-block with ordinal `stop` in a row that has more than `stop` of them; a converged warp, a lane per
 // word.
-__device__ __forceinline__ int kb_at_ordinal(const uint32_t* __restrict__ row, int i, int R, int T, int stop) {
+__device__ __forceinline__ int kb_at_ordinal(const uint32_t* row, int i, int R, int T, int stop) {
   const int lane = threadIdx.x & 31;
   for (int w0 = 0; w0 <= (i >> 5); w0 += 32) {
     const int w = w0 + lane;
@@ -370,7 +370,7 @@ plan_rows_kernel(const PrefillParams p, int4* __restrict__ items, int4* __restri
 // of plan_rows_kernel, which took 135 us with a thread per row, 1,396 instead of 1,489 us).
 constexpr int kCombineRows = 16;
 __global__ void __launch_bounds__(kCombineRows * 32)
-combine_parts_kernel(const PrefillParams p, const int4* __restrict__ splits) {
+combine_parts_kernel(const PrefillParams p, const int4* splits) {
   pdl_wait();
   pdl_trigger();
   const int4 sp = splits[blockIdx.x];

@@ -116,7 +116,7 @@ struct StepWalk<128> {
   bool two;                   // blocks of 256: two sub-blocks each
   __device__ __forceinline__ void load(int w0) {
     w = w0;
-    ahead = w0 <= (i >> 5) ? __ldg(row + w0) : 0u;
+    ahead = w0 <= (i >> 5) ? row[w0] : 0u;
   }
   __device__ __forceinline__ void next() {
     if (row == nullptr) {
@@ -171,8 +171,8 @@ struct StepWalk<64> {
   uint32_t f_cur;                               // flags of the current block (see kStepLast above)
   __device__ __forceinline__ void load(int w0) {
     w = w0;
-    aheadA = w0 <= (iA >> 5) ? __ldg(rowA + w0) : 0u;
-    aheadB = rowB && w0 <= (iB >> 5) ? __ldg(rowB + w0) : 0u;
+    aheadA = w0 <= (iA >> 5) ? rowA[w0] : 0u;
+    aheadB = rowB && w0 <= (iB >> 5) ? rowB[w0] : 0u;
   }
   __device__ __forceinline__ void next() {
     while ((ua | ub) == 0u) {
@@ -383,7 +383,7 @@ prefill_duo_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const int kvid = rem_band / per_band_kv;
         int rem = rem_band % per_band_kv;
         int4 item = make_int4(0, 0, 0x7fffffff, -1);
-        if (SCHED) { item = __ldg(p.items + w); rem = item.x; }
+        if (SCHED) { item = p.items[w]; rem = item.x; }
         const int l = kvid / Hkv, hk = kvid % Hkv;
         const int Tl = n_rows - 1 - (band * p.band_rows + rem / p.G);
         w = -2;

@@ -32,7 +32,7 @@ constexpr int kRankRows = kPrepThreads / 4;   // up to this many blocks are rank
 // launch that would share one sort; the counters of the scoring kernel are cleared here for the same reason (three
 // launches, a memset among them, in one).
 __global__ void __launch_bounds__(kPrepThreads)
-select_prep_kernel(const float* __restrict__ radius, const float* __restrict__ centroid, int M, int P /* pow2 >= M */,
+select_prep_kernel(const float* radius, const float* centroid, int M, int P /* pow2 >= M */,
                    float scale_log2, float* __restrict__ beta, float* __restrict__ rq, float* __restrict__ gs,
                    int* __restrict__ perm, __nv_bfloat16* __restrict__ chi, __nv_bfloat16* __restrict__ clo,
                    float* __restrict__ cnorm, int Mpad, int tiles_per_slice,
@@ -644,8 +644,8 @@ select_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // the row's constants are requested before the wait for the accumulator: their latency passes under it
         const int prow = crow0 + bt * 128 + row;
         const bool prow_ok = RBS_DBG_OK(prow >= 0 && prow < p.L * Hkv * p.Mpad, status, kDbgSelectCentroid);
-        const float gs = prow_ok ? __ldg(p.gs + prow) : 0.f, cn = prow_ok ? __ldg(p.cnorm + prow) : 0.f;
-        const int b_row = prow_ok ? __ldg(p.perm + prow) : 0x7fffffff;   // the block this accumulator row belongs to
+        const float gs = prow_ok ? p.gs[prow] : 0.f, cn = prow_ok ? p.cnorm[prow] : 0.f;
+        const int b_row = prow_ok ? p.perm[prow] : 0x7fffffff;   // the block this accumulator row belongs to
         ok = __all_sync(0xffffffffu, wait_accumulator(&bar_tfull[hw][buf], (nt >> 1) & 1));
         if (!ok) break;
         tc_fence_after_sync();
