@@ -24,6 +24,7 @@ CASES = [
     dict(name="dbg_b128", L=2, N=128 * 37 + 50, Hq=4, Hkv=2, B=128, sigma=(0.1, 1.0), seed=92),
     dict(name="dbg_b256", N=256 * 7 + 200, Hq=3, Hkv=1, B=256, sigma=(0.1, 1.0), s_q=3.5, seed=93),
     dict(name="dbg_split", N=128 * 300 + 77, Hq=2, Hkv=1, B=128, sigma=(0.1, 1.0), seed=94, n_recent=2),   # rows cut into parts
+    dict(name="dbg_split256", N=256 * 131 + 77, Hq=2, Hkv=1, B=256, sigma=(0.1, 1.0), seed=95, n_recent=1),
 ]
 
 CHILD = r"""
@@ -97,17 +98,23 @@ WAIT_CHILD = r"""
 import sys, time, torch
 from paper_2609_20971_b200 import rbs_sparse_prefill, rbs_device_status
 from paper_2609_20971_b200.binding import prefill_workspace_bytes, rbs_selftest_attention_wait
-N, Hq, Hkv = 64 * 80 - 20, 16, 2
 g = torch.Generator(device="cuda").manual_seed(5)
-Q, K, V = (torch.randn(1, N, h, 128, generator=g, device="cuda") for h in (Hq, Hkv, Hkv))
-K += 0.05 * torch.arange(N, device="cuda").view(1, N, 1, 1) / 64     # logits that grow: maxima go stale all the time
-Q += 0.5
-Q, K, V = Q.bfloat16(), K.bfloat16(), V.bfloat16()
-ws = torch.empty(prefill_workspace_bytes(1, N, Hq, Hkv, 128), dtype=torch.uint8, device="cuda")
+def problem(N, Hq, Hkv, slope):
+    Q, K, V = (torch.randn(1, N, h, 128, generator=g, device="cuda") for h in (Hq, Hkv, Hkv))
+    K += slope * torch.arange(N, device="cuda").view(1, N, 1, 1) / 64     # logits that grow: maxima go stale all the time
+    Q += 0.5
+    return Q.bfloat16(), K.bfloat16(), V.bfloat16()
+plain = problem(64 * 80 - 20, 16, 2, 0.05)
+cut = problem(128 * 260 - 20, 4, 2, 0.02)          # dense rows of more than 256 key tiles: planner, parts and merge
+ws = torch.empty(prefill_workspace_bytes(1, cut[0].shape[1], 4, 2, 128), dtype=torch.uint8, device="cuda")
 def call(B, schedule):
-    M = (N + B - 1) // B
-    mask = torch.full((1, Hq, M, (M + 31) // 32), -1, dtype=torch.int32, device="cuda")
-    return rbs_sparse_prefill(Q, K, V, mask, B, out=torch.zeros_like(Q), workspace=ws if schedule else None)
+    Q, K, V = cut if schedule else plain
+    M = (Q.shape[1] + B - 1) // B
+    mask = torch.full((1, Q.shape[2], M, (M + 31) // 32), -1, dtype=torch.int32, device="cuda")
+    ws.fill_(0x6B)
+    out = rbs_sparse_prefill(Q, K, V, mask, B, out=torch.zeros_like(Q), workspace=ws if schedule else None)
+    assert schedule == bool((ws != 0x6B).any())
+    return out
 want = {k: call(*k) for k in ((64, False), (128, False), (128, True))}
 assert rbs_device_status(clear=True) == 0
 for B, schedule, warp, which, before in eval(sys.argv[1]):
@@ -130,7 +137,7 @@ print("wait child ok")
 # maximum) and later ones, blocks of 64 with one and with two checks
 WAITS = [
     (128, False, 0, 0, 0), (128, False, 5, 0, 2), (128, False, 0, 1, 0), (128, False, 13, 1, 4), (128, False, 4, 2, 1),
-    (128, False, 9, 3, 0), (128, False, 0, 4, 0), (128, True, 6, 1, 2),
+    (128, False, 9, 3, 0), (128, False, 0, 4, 0), (128, True, 6, 1, 2), (128, True, 13, 0, 1), (128, True, 3, 4, 0), (128, True, 8, 3, 1),
     (64, False, 0, 0, 1), (64, False, 5, 1, 0), (64, False, 8, 1, 3), (64, False, 2, 2, 0), (64, False, 4, 2, 5),
     (64, False, 1, 3, 1), (64, False, 12, 4, 1),
 ]

@@ -8,6 +8,7 @@ from paper_2609_20971_b200 import alloc_stats, rbs_block_stats, rbs_device_statu
 from paper_2609_20971_b200.binding import RBS_OP_SELECT, RBS_OP_SPARSE_PREFILL, RbsShape
 
 pytestmark = pytest.mark.gpu
+FILL = 0x6B
 
 
 class _Problem:
@@ -21,7 +22,7 @@ class _Problem:
         self.density = torch.empty(1, Hq, dtype=torch.float32, device=dev)
         self.ws = torch.empty(max(256, workspace_bytes(RBS_OP_SELECT, shape)), dtype=torch.uint8, device=dev)
         n = workspace_bytes(RBS_OP_SPARSE_PREFILL, shape) if schedule else 0
-        self.ws_att = torch.empty(n, dtype=torch.uint8, device=dev) if n else None
+        self.ws_att = torch.full((n,), FILL, dtype=torch.uint8, device=dev) if n else None
 
     def fill(self, seed):
         g = torch.Generator(device="cuda").manual_seed(seed)
@@ -43,6 +44,7 @@ class _Problem:
 @pytest.mark.parametrize("first, second", [
     ((1003, 8, 2, 128, False), (64 * 21, 3, 1, 64, False)),
     ((256 * 9 + 100, 4, 1, 256, True), (128 * 150, 18, 6, 128, False)),
+    ((256 * 129 + 100, 4, 1, 256, True), (128 * 290 + 5, 6, 2, 128, True)),     # rows of more than 256 tiles: planner and merge
 ])
 def test_replays_of_a_graph_with_a_fork_and_a_join(first, second):
     a, b = _Problem(*first), _Problem(*second)
@@ -68,6 +70,9 @@ def test_replays_of_a_graph_with_a_fork_and_a_join(first, second):
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=main):
         both()
+    for p in (a, b):      # a workspace is written to where the longest row (the last one is dense) is long enough to be cut
+        tiles = p.mask.shape[2] * (p.B // 128)
+        assert p.ws_att is None or (tiles > 256) == bool((p.ws_att != FILL).any())
     for seed in (3, 5, 7):
         a.fill(seed), b.fill(seed + 1)
         dense.zero_()

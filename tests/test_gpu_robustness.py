@@ -44,12 +44,13 @@ def test_waits_of_a_whole_warp_give_every_lane_the_same_answer():
         assert rbs_device_status(clear=True) == WAIT_SELFTEST_CODE
 
 
-@pytest.mark.parametrize("B", [64, 128, 256])
-def test_a_recorded_time_out_leaves_later_calls_alone(B):
+@pytest.mark.parametrize("B, blocks", [(64, 21), (128, 21), (256, 21), (128, 261), (256, 131)])
+def test_a_recorded_time_out_leaves_later_calls_alone(B, blocks):
     """The status word belongs to the launch that wrote it: calls issued while it still holds a code give the bits they
-    give without one, and leave the code for whoever reads it."""
+    give without one, and leave the code for whoever reads it.  With 261 tiles of 128 and more a call with a workspace runs the
+    planner, the scheduled attention kernel and the merge."""
     from paper_2609_20971_b200.binding import prefill_workspace_bytes
-    cfg = SynthConfig("sticky", N=B * 21 + 37, Hq=4, Hkv=2, B=B, sigma=(0.1, 1.0), seed=91)
+    cfg = SynthConfig("sticky", N=B * blocks + 37, Hq=4, Hkv=2, B=B, sigma=(0.1, 1.0), seed=91)
     Q, K, V = (t.cuda() for t in make_inputs(cfg))
     ws = torch.empty(max(256, prefill_workspace_bytes(1, cfg.N, cfg.Hq, cfg.Hkv, B)), dtype=torch.uint8, device="cuda")
 
