@@ -308,7 +308,8 @@ def rbs_sparse_prefill(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, mask: 
                        workspace: torch.Tensor | None = None):
     """Causal block-sparse attention over `mask` (Sec. 3.3); mask=None is dense causal attention (Eq. 1).
     `workspace` (uint8, at least prefill_workspace_bytes(...)): opt into the row-length-aware schedule (blocks of 128
-    or 256): rows of more than 256 key tiles are cut into parts that run side by side and are merged afterwards."""
+    or 256): rows of more than 256 key tiles are cut into parts that run side by side and are merged afterwards.  Calls that
+    can have no such row leave the workspace alone."""
     lib = load_library()
     L, N, Hq, d = Q.shape
     shape = RbsShape(L, N, Hq, K.shape[2], d, block)

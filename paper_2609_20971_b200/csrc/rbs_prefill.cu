@@ -201,6 +201,9 @@ prefill_mma_kernel(const PrefillParams p) {
 // i.e. longest candidate range first, the G heads of a row together).  The first kSplitRowsPerGroup rows of that
 // order that exceed kSplitCap sub-blocks are cut into up to kSplitMaxParts parts of equal length, placed next to each
 // other.  (Sorting the rows of a group by their counts was measured as well: 0.03 - 0.1 ms slower on the 128K layer.)
+// One CTA per group, bound by the latency of the mask's words: a warp counts a row, a lane per word (selection and attention of
+// the last 64 query blocks of 128K tokens, 32 heads: the launch 22.6 us alone instead of 99 with a thread per row, the two calls
+// 1,326 instead of 1,399 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int kPlanThreads = 1024;
 
@@ -366,8 +369,8 @@ plan_rows_kernel(const PrefillParams p, int4* __restrict__ items, int4* __restri
 // (the maximum is only a shift, Sec. 3.3's softmax over the retained keys is unchanged), parts taken in order.
 // One CTA per (group, split-row slot, 16 query rows), a warp per row: bound by the latency of two dependent loads per row,
 // so that all of a CTA's rows are on their way together (the last 64 query blocks of 128K tokens of 32 heads, 32 split rows:
-// 69 us with 32 CTAs of four warps that take one row after the other; a whole pass over that chunk, with the warp-wide counting
-// of plan_rows_kernel, which took 135 us with a thread per row, 1,396 instead of 1,489 us).
+// the launch 5.5 us alone instead of 55 with 32 CTAs of four warps that take one row after the other; selection and attention
+// 1,280 instead of 1,326 us, and 1,267 with planner and merge as dependent launches).
 constexpr int kCombineRows = 16;
 __global__ void __launch_bounds__(kCombineRows * 32)
 combine_parts_kernel(const PrefillParams p, const int4* splits) {
@@ -437,9 +440,12 @@ static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q,
   rbs_status st;
   PrefillParams pp = p;
   const int n_rows = p.Mq * p.R;
-  // the schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink
-  // steadily), rows long enough to be cut (a row that is not cut gives the same bits either way; selection and attention of
-  // 2K of 8K tokens, 32 heads: 125 us without planner and merge, 153 with them) and a group whose counts fit the planner's shared memory
+  // The schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink steadily), a
+  // group whose counts fit the planner's shared memory, and rows long enough to be cut: a row of kSplitCap sub-blocks or fewer
+  // gives the same bits either way, planner and merge are lost on it, and small K/V lose the order by rows (tile_bands).
+  // Attention of 32 heads with the schedule /
+  // without: 1,003 tokens 27.4 / 19.3 us, the last 2K of 8K 129.7 / 98.2, 8K 228 / 178, the last 2K of 16K 222 / 174 - 199, the last
+  // 2K of 32K (256 sub-blocks, the longest that this sends the plain way) 411 - 443 / 395 - 437, 32K 1,404 - 1,434 / 1,387 - 1,409.
   const double kv_bytes = 4.0 * kHeadDim * p.L * Hkv * static_cast<double>(p.N);
   const int sched_bands = tile_bands(n_rows, true, 0.0);
   const bool scheduled = p.mask != nullptr && workspace != nullptr && (p.q0 + p.Mq) * p.R > kSplitCap &&

@@ -29,11 +29,12 @@ struct PrefillParams {
 };
 
 // Rows longer than this many 128-key sub-blocks are cut into parts of equal length that run as separate CTAs and are
-// merged afterwards; the cut depends only on the row itself, so a row is treated the same in every call.
+// merged afterwards.  How a row is cut depends only on the row; whether it is, also on the group: its first
+// kSplitRowsPerGroup long rows are, counted from the end of its band of the call's queries.
 constexpr int kSplitCap = 256;
 constexpr int kSplitMaxParts = 4;      // parts per split row
 constexpr int kMaxBands = 4;           // bands of the scheduled tile order
-constexpr int kSplitRowsPerGroup = 8;  // split rows per (band, batch, KV head) group: its longest ones
+constexpr int kSplitRowsPerGroup = 8;  // split rows per (band, batch, KV head) group: its last ones in the sequence
 constexpr int kSplitSlotsPerGroup = kSplitRowsPerGroup * kSplitMaxParts;
 constexpr int kExtraItemsPerGroup = kSplitRowsPerGroup * (kSplitMaxParts - 1);
 

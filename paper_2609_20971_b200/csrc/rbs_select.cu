@@ -19,7 +19,7 @@ namespace rbs {
 //    with zeros
 // ---------------------------------------------------------------------------------------------
 constexpr int kPrepThreads = 1024;
-constexpr int kRankRows = kPrepThreads / 4;   // up to this many blocks are ranked by counting
+constexpr int kRankRows = kPrepThreads / 4;   // up to this many blocks are ranked by counting: four threads per block
 
 // Besides beta, the kernel fixes the ORDER in which the scoring kernels see the blocks of each 128-row centroid tile:
 // inside a tile the rows with r_b beta_b = 0 (at least half of all blocks: every radius at or below the median) come
@@ -52,10 +52,11 @@ select_prep_kernel(const float* radius, const float* centroid, int M, int P /* p
   }
   const float* r = radius + static_cast<int64_t>(hd) * M;
   if (M <= kRankRows) {
-    // Few blocks: bound by the latency of the sort's passes, a barrier each (21 at 64 blocks).  Every radius counts the
-    // ones in front of it instead, four threads per radius (an order-preserving integer image: NaN has a place too).  Whole
-    // passes, sorted / counted: 4K tokens of one head at blocks of 64 (64 blocks) 69.7 / 67.0 us, twelve packed prompts of
-    // 3 to 125 blocks 1,405 / 1,394, 1,003 tokens of 32 heads (8 blocks) the same.
+    // Few blocks: bound by the latency of the sort's passes, a barrier each (21 at 64 blocks, 36 at 256).  Every radius
+    // counts the ones in front of it instead, four threads per radius (an order-preserving integer image: NaN has a place
+    // too).  rbs_select call after call, sorted / counted, blocks of 64: one head, 33 blocks 15.9 / 14.0 us, 64 15.8 / 13.6,
+    // 129 19.7 / 15.2, 256 21.0 / 17.6; 32 heads, 8 blocks 22.1 / 22.1, 64 39.3 / 37.1, 129 63.0 / 58.4, 256 135.4 / 131.6.
+    // It pays up to the limit, which is where the threads run out.
     const int idx = tid >> 2, part = tid & 3;
     if (tid < kRankRows) {
       const uint32_t u = tid < M ? __float_as_uint(r[tid]) : 0xffffffffu;
@@ -71,21 +72,21 @@ select_prep_kernel(const float* radius, const float* centroid, int M, int P /* p
     if (part == 0 && idx < M) s_sorted[rank] = r[idx];
     __syncthreads();
   } else {
-  for (int idx = tid; idx < P; idx += kPrepThreads) s_sorted[idx] = idx < M ? r[idx] : __int_as_float(0x7f800000);
-  __syncthreads();
-  for (int k = 2; k <= P; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int idx = tid; idx < P; idx += kPrepThreads) {
-        const int ixj = idx ^ j;
-        if (ixj > idx) {
-          const float a = s_sorted[idx], c = s_sorted[ixj];
-          const bool asc = (idx & k) == 0;
-          if ((a > c) == asc) { s_sorted[idx] = c; s_sorted[ixj] = a; }
+    for (int idx = tid; idx < P; idx += kPrepThreads) s_sorted[idx] = idx < M ? r[idx] : __int_as_float(0x7f800000);
+    __syncthreads();
+    for (int k = 2; k <= P; k <<= 1) {
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int idx = tid; idx < P; idx += kPrepThreads) {
+          const int ixj = idx ^ j;
+          if (ixj > idx) {
+            const float a = s_sorted[idx], c = s_sorted[ixj];
+            const bool asc = (idx & k) == 0;
+            if ((a > c) == asc) { s_sorted[idx] = c; s_sorted[ixj] = a; }
+          }
         }
+        __syncthreads();
       }
-      __syncthreads();
     }
-  }
   }
   if (tid < 2) {
     // quantile(p): linear interpolation between order statistics at position p (M - 1)

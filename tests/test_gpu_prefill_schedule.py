@@ -114,3 +114,39 @@ def test_rows_at_the_edge_of_the_schedule(block, m, q0, rows):
             ref, lref = torch.softmax(x, -1) @ v[0, keys, g].double(), torch.logsumexp(x, -1)
             assert ((a.double() - ref).norm() / ref.norm()).item() <= 6.4e-3
             assert (la.double() - lref).abs().max().item() <= 1e-4
+
+
+def test_calls_in_a_row_plan_from_the_mask_of_their_own_selection():
+    """Selection and scheduled attention of two prompts by turns, in one mask, one workspace and without a pause between them,
+    as an engine issues them: the planner may become resident while the selector still writes the mask, and the next
+    call's kernels while the merge still runs."""
+    from paper_2609_20971_b200 import rbs_block_stats, rbs_select, rbs_sparse_prefill, workspace_bytes
+    from paper_2609_20971_b200.binding import RBS_OP_SELECT, RBS_OP_SPARSE_PREFILL, RbsShape
+    n, hq, hkv, block = 128 * 290 - 40, 8, 2, 128
+    shape, gen = RbsShape(1, n, hq, hkv, 128, block), torch.Generator(device="cuda").manual_seed(9)
+    prompts = []
+    for scale in (1.0, 2.5):                             # different densities: other rows are long
+        coherent = torch.randn(1, 290, hq, 128, generator=gen, device="cuda").repeat_interleave(block, 1)[:, :n]
+        q = scale * (torch.randn(1, n, hq, 128, generator=gen, device="cuda") + coherent)
+        k, v = (torch.randn(1, n, hkv, 128, generator=gen, device="cuda").bfloat16() for _ in range(2))
+        prompts.append((q.bfloat16(), k, v, rbs_block_stats(k, block)))
+    mask = torch.empty(1, hq, 290, 10, dtype=torch.int32, device="cuda")
+    ws = torch.empty(workspace_bytes(RBS_OP_SELECT, shape), dtype=torch.uint8, device="cuda")
+    ws_att = torch.empty(workspace_bytes(RBS_OP_SPARSE_PREFILL, shape), dtype=torch.uint8, device="cuda")
+
+    def call(x, out):
+        q, k, v, stats = prompts[x]
+        rbs_select(q, stats, block, n_recent=2, mask=mask, workspace=ws)
+        rbs_sparse_prefill(q, k, v, mask, block, out=out, workspace=ws_att)
+    want, masks = [torch.empty_like(prompts[0][0]) for _ in range(2)], []
+    for x in range(2):
+        call(x, want[x])
+        torch.cuda.synchronize()
+        masks.append(mask.clone())
+    assert not torch.equal(*masks)
+    outs = [torch.zeros_like(want[0]) for _ in range(12)]
+    torch.cuda.synchronize()
+    for x, out in enumerate(outs):
+        call(x % 2, out)
+    torch.cuda.synchronize()
+    assert all(torch.equal(out, want[x % 2]) for x, out in enumerate(outs))
