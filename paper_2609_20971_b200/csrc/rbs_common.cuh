@@ -138,6 +138,14 @@ inline cudaError_t launch_pdl(void (*kernel)(KernelArgs...), unsigned grid_x, un
 // what another kernel of the path wrote (mask, items, statistics, scratch) is never read that way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A plain load that stays behind pdl_wait (both are volatile) and is free to pass the stores around it.  For the mask words of a
+// producer's walk: attention of 64 heads over 128K tokens at blocks of 64, 12 runs in turn, 23,668 us with `row[w]`, 23,601 with
+// this, 23,614 with the non-coherent load (runs of one side differ by 26).
+__device__ __forceinline__ uint32_t load_written(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
 
 #define RBS_CUDA_OK(expr)                               \
   do {                                                  \

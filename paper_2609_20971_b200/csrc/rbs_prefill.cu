@@ -443,9 +443,9 @@ static rbs_status launch_prefill_tc(const PrefillParams& p, const rbs_tensor& Q,
   // The schedule needs the mask (dense attention keeps its tiles whole: its launch is long and its rows shrink steadily), a
   // group whose counts fit the planner's shared memory, and rows long enough to be cut: a row of kSplitCap sub-blocks or fewer
   // gives the same bits either way, planner and merge are lost on it, and small K/V lose the order by rows (tile_bands).
-  // Attention of 32 heads with the schedule /
-  // without: 1,003 tokens 27.4 / 19.3 us, the last 2K of 8K 129.7 / 98.2, 8K 228 / 178, the last 2K of 16K 222 / 174 - 199, the last
-  // 2K of 32K (256 sub-blocks, the longest that this sends the plain way) 411 - 443 / 395 - 437, 32K 1,404 - 1,434 / 1,387 - 1,409.
+  // Attention of 32 heads with the schedule / without: 1,003 tokens 27.4 / 19.3 us, the last 2K of 8K 129.7 / 98.2, 8K 228 / 178,
+  // the last 2K of 16K 222 / 174 - 199, the last 2K of 32K (256 sub-blocks, the longest that goes the plain way) 411 - 443 /
+  // 395 - 437, 32K 1,404 - 1,434 / 1,387 - 1,409.
   const double kv_bytes = 4.0 * kHeadDim * p.L * Hkv * static_cast<double>(p.N);
   const int sched_bands = tile_bands(n_rows, true, 0.0);
   const bool scheduled = p.mask != nullptr && workspace != nullptr && (p.q0 + p.Mq) * p.R > kSplitCap &&

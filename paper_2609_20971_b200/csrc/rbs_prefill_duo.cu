@@ -116,7 +116,7 @@ struct StepWalk<128> {
   bool two;                   // blocks of 256: two sub-blocks each
   __device__ __forceinline__ void load(int w0) {
     w = w0;
-    ahead = w0 <= (i >> 5) ? row[w0] : 0u;
+    ahead = w0 <= (i >> 5) ? load_written(row + w0) : 0u;
   }
   __device__ __forceinline__ void next() {
     if (row == nullptr) {
@@ -171,8 +171,8 @@ struct StepWalk<64> {
   uint32_t f_cur;                               // flags of the current block (see kStepLast above)
   __device__ __forceinline__ void load(int w0) {
     w = w0;
-    aheadA = w0 <= (iA >> 5) ? rowA[w0] : 0u;
-    aheadB = rowB && w0 <= (iB >> 5) ? rowB[w0] : 0u;
+    aheadA = w0 <= (iA >> 5) ? load_written(rowA + w0) : 0u;
+    aheadB = rowB && w0 <= (iB >> 5) ? load_written(rowB + w0) : 0u;
   }
   __device__ __forceinline__ void next() {
     while ((ua | ub) == 0u) {
