@@ -130,17 +130,18 @@ RBS_API rbs_status rbs_select(const rbs_shape* shape, rbs_tensor Q, rbs_stats st
  * softmax_scale == 0 means 1/sqrt(d).
  * Workspace: optional (NULL / 0: none).  With mask != NULL, block >= 128 and a workspace of at least
  * rbs_workspace_bytes(RBS_OP_SPARSE_PREFILL, shape) bytes (256-byte aligned; RBS_ERR_WORKSPACE if too small or
- * misaligned) a call whose longest possible row, that of its last query block, has more than 256 key tiles of 128 (shorter
- * calls leave the workspace alone and give the bits of a call without one) derives a schedule from the mask first --
- * per-row counts of selected blocks, rows of more than 256 key tiles cut into up to 4 parts of equal length (the index
- * compaction of Sec. 3.3's cost paragraph, O(M K_avg) entries, reduced to what the kernel needs) -- runs the parts as
- * separate thread blocks and merges their partial results in a fixed order (bitwise repeatable).  A row here is 128 queries
- * of one head; of each KV head the last 8 such rows of the call are cut (in calls of 128 rows per head and more the last 8
- * of each band of rows, two to four bands), in a way that depends only on the row.  So a row gives the same bits in a whole-sequence call and in any chunked call that is also
- * given a workspace, unless a KV head has more than 8 such rows and the two calls cut different ones; a row that is cut in
- * only one of two calls agrees to rounding.  This pays when a call is short next to its longest rows, as chunked calls are
- * (attention of the last 64 query blocks of a 128K layer, 32 heads: 1.07 against 1.96 - 2.11 ms; of the last 16: 0.54 against
- * 1.54); on a whole 128K layer it makes no difference.
+ * misaligned) a call whose last query block has more than 256 key tiles of 128 derives a schedule from the mask first --
+ * per-row counts of selected blocks (a row is 128 queries of one head), rows of more than 256 selected tiles cut into up
+ * to 4 parts of equal length (the index compaction of Sec. 3.3's cost paragraph, O(M K_avg) entries, reduced to what the
+ * kernel needs) -- runs the parts as separate thread blocks and merges their partial results in a fixed order (bitwise
+ * repeatable).  Shorter calls leave the workspace alone and give the bits of a call without one.
+ * Of each KV head the last 8 such rows of the call are cut (where a head has 128 rows or more in the call: the last 8 of
+ * each of two to four bands of rows); how depends only on the row.  So a row gives the same bits in a whole-sequence call
+ * and in any chunked call that is also given a workspace, unless a KV head has more than 8 such rows and the two calls
+ * cut different ones; a row that is cut in only one of two calls agrees to rounding.
+ * This pays when a call is short next to its longest rows, as chunked calls are (attention of the last 64 query blocks of
+ * a 128K layer, 32 heads: 1.07 against 1.96 - 2.11 ms; of the last 16: 0.54 against 1.54); on a whole 128K layer it makes
+ * no difference.
  * The size depends on the shape only: one buffer serves the whole-sequence call and every chunked call.
  */
 RBS_API rbs_status rbs_sparse_prefill(const rbs_shape* shape, rbs_tensor Q, rbs_tensor K, rbs_tensor V,
